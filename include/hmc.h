@@ -352,7 +352,7 @@ int hmc_rng_draw(uint64_t seed, uint32_t stream_id, uint64_t traj, uint32_t chai
  * the device heap -- cannot create an hmc_ctx.  This call needs none: it
  * runs the same FP64 CG as hmc_cg_solve with HMC_PREC_FP64 (same algorithm,
  * stopping rule and stats), with its scratch in one static device array of
- * about 2.1 MB that every GPU which loads the library holds until the
+ * about 2.9 MB that every GPU which loads the library holds until the
  * process exits.
  *
  *   E      device, double [V][V], the transfer matrix exp(delta*kappa*h),
@@ -370,7 +370,7 @@ int hmc_rng_draw(uint64_t seed, uint32_t stream_id, uint64_t traj, uint32_t chai
  * array's device address (cudaGetSymbolAddress) with that device current.
  * Every call on a device shares the one array: calls that overlap on the
  * GPU (other streams, other host threads) race and give wrong results;
- * serialise them.  The barrier, status and output words are cleared on
+ * serialise them.  The status, output and team words are cleared on
  * every call.  Errors as hmc_cg_solve. */
 int hmc_cg_solve_noalloc(const double* E, int L, int Nt, const double* phi, const void* chi,
                          void* x, double tol, int max_iter, hmc_cg_stats* stats, void* stream);

@@ -208,6 +208,8 @@ int hmc_ctx_create(const hmc_params* p, hmc_ctx** out) {
         const double f = std::exp(-v.delta * p->mu);
         for (double& e : E) e *= f;
     }
+    hop_series_build(p->L, v.delta * p->kappa, p->mu != 0.0 ? std::exp(-v.delta * p->mu) : 1.0,
+                     &v.ser);
     bool ok = true;
     const size_t N = (size_t)v.N;
     double* dE = (double*)ctx_alloc(c, E.size() * sizeof(double), &ok);
@@ -215,6 +217,7 @@ int hmc_ctx_create(const hmc_params* p, hmc_ctx** out) {
     v.x = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
     v.r = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
     v.p = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
+    v.p2 = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
     v.q = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
     v.chi = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
     v.rho = (double2*)ctx_alloc(c, N * sizeof(double2), &ok);
@@ -226,10 +229,7 @@ int hmc_ctx_create(const hmc_params* p, hmc_ctx** out) {
     }
     v.pi = (double*)ctx_alloc(c, N * sizeof(double), &ok);
     v.phi_old = (double*)ctx_alloc(c, N * sizeof(double), &ok);
-    v.bar = (unsigned*)ctx_alloc(c, 8 * sizeof(unsigned), &ok);
-    v.status = (int*)ctx_alloc(c, kStatusBlockBytes, &ok);
-    v.partials = (double*)ctx_alloc(c, sizeof(double) * kPartialDoubles, &ok);
-    v.scalars = (double*)ctx_alloc(c, sizeof(double) * kNumScalars, &ok);
+    control_bind(&v, ctx_alloc(c, kControlBytes, &ok));
     if (ok && cudaMemcpy(dE, E.data(), E.size() * sizeof(double), cudaMemcpyHostToDevice) !=
                   cudaSuccess)
         ok = false;
@@ -270,11 +270,8 @@ static int apply_common(hmc_ctx* c, const double* phi, const void* in, void* out
                         void* stream, bool dag) {
     if (!c || !phi || !in || !out || in == out) return HMC_ERR_BAD_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (prec == HMC_PREC_FP64) {
-        int st = launch_cis_f64(c->view, phi, s);
-        if (st != HMC_OK) return st;
-        return launch_apply_f64(c->view, dag, (const double2*)in, (double2*)out, s);
-    }
+    if (prec == HMC_PREC_FP64)
+        return launch_apply_f64(c->view, dag, phi, (const double2*)in, (double2*)out, s);
     if (prec == HMC_PREC_MIXED) return tc_apply(c, phi, (const float2*)in, (float2*)out, dag, s);
     return HMC_ERR_BAD_ARG;
 }
@@ -295,10 +292,6 @@ int hmc_cg_solve(hmc_ctx* c, const double* phi, const void* chi, void* x, double
     if (!(tol > 0.0) || max_iter < 1) return HMC_ERR_BAD_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     std::memset(stats, 0, sizeof(*stats));
-    if (cudaMemsetAsync(c->view.status, 0, sizeof(int), s) != cudaSuccess ||
-        cudaMemsetAsync(c->view.bar, 0, 8 * sizeof(unsigned), s) != cudaSuccess ||
-        cudaMemsetAsync(c->view.scalars, 0, sizeof(double) * kNumScalars, s) != cudaSuccess)
-        return HMC_ERR_CUDA;
     int st;
     if (prec == HMC_PREC_FP64)
         st = launch_cg_f64(c->view, c->num_sms, phi, (const double2*)chi, (double2*)x, tol,
@@ -328,8 +321,6 @@ int hmc_cg_solve(hmc_ctx* c, const double* phi, const void* chi, void* x, double
 int hmc_force(hmc_ctx* c, const double* phi, const void* x, double* F, void* stream) {
     if (!c || !phi || !x || !F) return HMC_ERR_BAD_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    int st = launch_cis_f64(c->view, phi, s);
-    if (st != HMC_OK) return st;
     return launch_force_f64(c->view, phi, (const double2*)x, F, s);
 }
 
@@ -352,10 +343,6 @@ int hmc_trajectory(hmc_ctx* c, double* phi, uint64_t seed, uint64_t traj_index, 
     if (!c || !phi || !out) return HMC_ERR_BAD_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     std::memset(out, 0, sizeof(*out));
-    if (cudaMemsetAsync(c->view.status, 0, sizeof(int), s) != cudaSuccess ||
-        cudaMemsetAsync(c->view.bar, 0, 8 * sizeof(unsigned), s) != cudaSuccess ||
-        cudaMemsetAsync(c->view.scalars, 0, sizeof(double) * kNumScalars, s) != cudaSuccess)
-        return HMC_ERR_CUDA;
     TrajArgs a;
     a.phi = phi;
     a.seed = seed;
@@ -405,7 +392,7 @@ int hmc_ctx_set_wait_limit(hmc_ctx* c, double seconds) {
     if (!c || !(seconds >= 0.0) || seconds > 3600.0) return HMC_ERR_BAD_ARG;
     const uint64_t ns = (uint64_t)(seconds * 1e9);
     if (cudaDeviceSynchronize() != cudaSuccess ||
-        cudaMemcpy(c->view.status + 2, &ns, sizeof(ns), cudaMemcpyHostToDevice) != cudaSuccess)
+        cudaMemcpy(c->view.status - 2, &ns, sizeof(ns), cudaMemcpyHostToDevice) != cudaSuccess)
         return HMC_ERR_CUDA;
     return HMC_OK;
 }

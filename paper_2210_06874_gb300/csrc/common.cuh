@@ -4,10 +4,9 @@
 #pragma once
 
 #include <cuda_runtime.h>
-#include <cuda/atomic>
 #include <stdint.h>
 
-#include "../../include/hmc.h"
+#include "ctx.h"
 
 namespace hmc {
 
@@ -78,25 +77,21 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // Every spin in this library gives up after a time limit and records
-// HMC_ERR_TIMEOUT instead of waiting forever.  The limit lives in the
-// status block next to the status word: int status, int (unused), uint64
-// limit in ns at byte offset 8; zero there selects the default below.
+// HMC_ERR_TIMEOUT instead of waiting forever.  The limit (uint64, ns) lives
+// in the control block right before the status word; zero there selects the
+// default below.
 constexpr uint64_t kWaitLimitNs = 20ull * 1000ull * 1000ull * 1000ull;  // 20 s
-constexpr size_t kStatusBlockBytes = 16;
 __device__ __forceinline__ uint64_t wait_limit_ns(const int* status) {
-    const uint64_t v = *reinterpret_cast<const volatile uint64_t*>(status + 2);
+    const uint64_t v = *reinterpret_cast<const volatile uint64_t*>(status - 2);
     return v ? v : kWaitLimitNs;
 }
 
 // ---------------------------------------------------------------- team
 // A team is a set of co-resident CTAs of one persistent (cooperative)
-// launch that work on one Markov chain.  bar[0] = arrival count,
-// bar[1] = generation.  partials: per-CTA partial sums [kMaxTeam][kVals],
-// followed by the published team totals [kVals].
-constexpr int kMaxTeam = 1024;
+// launch that work on one Markov chain.  A global-memory team exchanges its
+// partial sums through sequence-tagged slots, one per CTA (control block in
+// ctx.h; cleared before every launch).
 constexpr int kVals = 4;
-constexpr int kSlots = 1;          // partial-sum buffers (one suffices, see team_sum)
-constexpr size_t kPartialDoubles = (size_t)kMaxTeam * kVals + kVals;
 
 // Synchronisation state of a team that is one thread-block cluster: every
 // CTA pushes its partial sums into every member's slot (distributed shared
@@ -124,9 +119,9 @@ struct ClusterSync {
 struct Team {
     int rank;          // CTA rank within the team
     int size;          // number of CTAs in the team
-    unsigned* bar;     // 2 words, zero-initialised
     int* status;       // shared device status word (hmc_status, 0 = ok)
-    double* partials;  // kPartialDoubles
+    uint64_t* slots;   // this team's words of rank 0's slot (rank r: + r kSlotWords)
+    unsigned* gen;     // shared memory: syncs this CTA has completed on the slots
     ClusterSync* cs;   // non-null: the team is this CTA's cluster, rank = cluster rank
 };
 
@@ -138,10 +133,92 @@ __device__ __forceinline__ void set_status(int* status, int code) {
     atomicCAS(status, 0, code);
 }
 
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
+// A double as two tagged words: each 64-bit word carries half the bits and the
+// sequence number, so a reader that sees both tags has the whole value.
+__device__ __forceinline__ void st_tagged(uint64_t* p, double v, unsigned seq) {
+    const uint64_t b = (uint64_t)__double_as_longlong(v), t = (uint64_t)seq << 32;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n\tst.relaxed.gpu.global.u64 [%0 + 8], %2;" ::
+                     "l"(p), "l"(t | (b & 0xffffffffull)), "l"(t | (b >> 32))
+                 : "memory");
+}
+__device__ __forceinline__ bool ld_tagged(const uint64_t* p, unsigned seq, double& v) {
+    uint64_t lo, hi;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%2];\n\tld.relaxed.gpu.global.u64 %1, [%2 + 8];"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+    v = __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
+    return (unsigned)(lo >> 32) == seq && (unsigned)(hi >> 32) == seq;
+}
+
+// Warp 0: post this CTA's NV values (valid on lane 0) under sequence number
+// seq, wait (bounded) for every member's, and sum them in rank order (lane r,
+// r + 32, ..., then a fixed shuffle tree); totals valid on lane 0.  One hop:
+// every CTA reads every slot.  A counter whose last arriver sums, publishes
+// and flips a generation word takes three dependent trips to L2 and four
+// fences; with 64 CTAs that barrier measured about 9 us, this one 2.
+// Buffers alternate: a CTA posts sync k + 2 only after sync k + 1, which
+// nobody posts before having read all of sync k.
+template <int NV, bool kF32>
+__device__ inline bool slot_sync(const Team& tm, unsigned seq, double* v) {
+    const int lane = threadIdx.x & 31;
+    uint64_t* const mine = tm.slots + (seq & 1u) * (2 * kVals);
+    if (lane == 0) {
+        __threadfence();   // release the block's writes (ordered before by its barrier)
+#pragma unroll
+        for (int j = 0; j < (NV > 0 ? NV : 1); ++j)
+            st_tagged(mine + (size_t)tm.rank * kSlotWords + 2 * j, NV > 0 ? v[j] : 0.0, seq);
+    }
+    __syncwarp();
+    bool ok = true;
+    const int size = min(tm.size, kMaxTeam);
+    constexpr int kInFlight = 8;
+#pragma unroll
+    for (int j = 0; j < (NV > 0 ? NV : 1); ++j) {
+        double a = 0.0;
+        for (int base = 0; base < size; base += 32 * kInFlight) {
+            double x[kInFlight];
+            uint64_t t0 = 0;
+            for (unsigned n = 1;; ++n) {
+                bool all = true;
+#pragma unroll
+                for (int i = 0; i < kInFlight; ++i) {
+                    const int r = base + lane + 32 * i;
+                    x[i] = 0.0;
+                    if (r < size)
+                        all = ld_tagged(mine + (size_t)r * kSlotWords + 2 * j, seq, x[i]) && all;
+                }
+                if (__all_sync(0xffffffffu, all || !ok)) break;
+                if ((n & 255u) == 0) {
+                    if (t0 == 0) t0 = global_ns();
+                    if (team_failed(tm)) ok = false;
+                    else if (global_ns() - t0 > wait_limit_ns(tm.status)) {
+                        set_status(tm.status, HMC_ERR_TIMEOUT);
+                        ok = false;
+                    }
+                }
+            }
+            if (NV > 0) {
+#pragma unroll
+                for (int i = 0; i < kInFlight; ++i)
+                    if (base + 32 * i < size) {
+                        if constexpr (kF32) a = (double)((float)a + (float)x[i]);
+                        else a += x[i];
+                    }
+            }
+        }
+        if (NV > 0) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double b = __shfl_down_sync(0xffffffffu, a, o);
+                if constexpr (kF32) a = (double)((float)a + (float)b);
+                else a += b;
+            }
+            v[j] = a;
+        }
+    }
+    __threadfence();   // acquire: the block's reads after its next barrier
+    return __all_sync(0xffffffffu, ok);
 }
 
 // Fixed-order CTA reduction of NV doubles; result valid on thread 0.
@@ -280,13 +357,8 @@ __device__ inline bool cluster_push_wait(const Team& tm, const double* v, float 
 }
 
 // Team barrier fused with a deterministic sum of NV values (NV = 0: plain
-// barrier).  Every CTA writes its partials, then arrives on the counter; the
-// last CTA to arrive sums the partials of all ranks in rank order (a fixed
-// order, so every run and every CTA gets the same bits), publishes the
-// totals and flips the generation word; the others spin (bounded) on the
-// generation and read the totals.  One buffer suffices: a CTA can write its
-// next partials only after passing this barrier, and the last arriver has
-// read every partial before it releases the barrier.
+// barrier): every CTA's block sum, added over the ranks in a fixed order, so
+// every run and every CTA gets the same bits.
 // Returns false on every thread of the CTA if the team failed or a wait
 // timed out.
 // kPre: the CTA's values are already summed and valid on thread 0 only.
@@ -343,72 +415,16 @@ __device__ inline bool team_sync(Team& tm, double* v) {
         __syncthreads();
         return ok != 0;
     }
-    double* totals = tm.partials + (size_t)kMaxTeam * kVals;
-    cuda::atomic_ref<unsigned, cuda::thread_scope_device> cnt(tm.bar[0]);
-    cuda::atomic_ref<unsigned, cuda::thread_scope_device> gen(tm.bar[1]);
-    unsigned g = 0;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) tm.partials[tm.rank * kVals + j] = v[j];
-        g = gen.load(cuda::memory_order_relaxed);
-        __threadfence();
-        s_last = cnt.fetch_add(1u, cuda::memory_order_acq_rel) == (unsigned)(tm.size - 1);
-    }
-    __syncthreads();
-    if (s_last) {
-        // last arriver: fixed-order sum of all partials by warp 0, publish
-        if (NV > 0 && threadIdx.x < 32) {
-            __threadfence();
-            const int lane = threadIdx.x;
-#pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                if constexpr (kF32) {
-                    float a = 0.f;
-                    for (int r = lane; r < tm.size; r += 32)
-                        a += (float)((volatile double*)tm.partials)[r * kVals + j];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-                    if (lane == 0) {
-                        totals[j] = (double)a;
-                        s_out[j] = (double)a;
-                    }
-                } else {
-                    double a = 0.0;
-                    for (int r = lane; r < tm.size; r += 32)
-                        a += ((volatile double*)tm.partials)[r * kVals + j];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-                    if (lane == 0) {
-                        totals[j] = a;
-                        s_out[j] = a;
-                    }
-                }
-            }
-        }
-        __syncthreads();
+    if constexpr (NV == 0) __syncthreads();   // the block's writes before the post
+    if (threadIdx.x < 32) {
+        const unsigned seq = *tm.gen + 1u;
+        const bool ok = slot_sync<NV, kF32>(tm, seq, v);
         if (threadIdx.x == 0) {
-            cnt.store(0u, cuda::memory_order_relaxed);
-            __threadfence();
-            gen.store(g + 1u, cuda::memory_order_release);
-            s_ok = !team_failed(tm);
-        }
-    } else if (threadIdx.x == 0) {
-        int ok = 1;
-        const uint64_t t0 = global_ns();
-        for (unsigned n = 1; ld_acquire_u32(&tm.bar[1]) == g; ++n) {
-            if ((n & 1023u) == 0) {
-                if (team_failed(tm)) { ok = 0; break; }
-                if (global_ns() - t0 > wait_limit_ns(tm.status)) {
-                    set_status(tm.status, HMC_ERR_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
+            *tm.gen = seq;
 #pragma unroll
-        for (int j = 0; j < NV; ++j) s_out[j] = ((volatile double*)totals)[j];
-        s_ok = ok && !team_failed(tm);
+            for (int j = 0; j < NV; ++j) s_out[j] = v[j];
+            s_ok = ok ? 1 : 0;
+        }
     }
     __syncthreads();
 #pragma unroll

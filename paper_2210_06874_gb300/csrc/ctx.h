@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/hmc.h"
+#include "series.h"
 
 namespace hmc {
 
@@ -15,6 +16,7 @@ struct ChainView {
     int L, V, Nt, N;            // N = V * Nt
     double delta, kappa, U;
     const double* E;            // V x V FP64, row-major, exactly symmetric
+    HopSeries ser;              // E as a polynomial of h (ser.ok = 0: only the dense E)
     // FP16 split of E for the tensor-core path (row-major, padded):
     //   E ~= (E_hi + E_lo * 2^-kLoShift) with rows and cols padded to Vp.
     const void* E_hi;           // __half [Vr][Vp]
@@ -28,6 +30,7 @@ struct ChainView {
     // FP64 workspaces, double2 [Nt][V] each
     double2 *cis;               // exp(i phi)
     double2 *x, *r, *p, *q, *chi, *rho;
+    double2 *p2;                // the CG direction's second buffer
     double2 *xh;                // solution history for the mixed trajectory's guesses
     double2 *chi2, *phi2, *x2;  // mass preconditioning: second pseudofermion, M_g chi2,
                                 // and its solve (allocated when hb_inner > 0)
@@ -50,15 +53,42 @@ struct ChainView {
     // rows, 128-byte swizzle); null when the context has no split-K shape
     const void* sk_maps;
     unsigned long long* gslots; // sequence-numbered partial sums and totals (tc_splitk.cuh)
-    // team synchronisation
-    unsigned* bar;              // 2 words
-    int* status;                // device status block (kStatusBlockBytes): status
-                                // word, then the wait limit (common.cuh)
+    // control block (control_bind below): wait limit, status word, outputs of
+    // the call, team slots
+    int* status;
+    double* scalars;            // per-call scalar outputs (see kernels)
+    uint64_t* slots;            // [kMaxTeam][kSlotWords] tagged partial sums
     int team_pad;               // testing only: CTAs every team barrier expects
                                 // beyond those launched (0 in normal use)
-    double* partials;           // kSlots * kMaxTeam * kVals
-    double* scalars;            // per-call scalar outputs (see kernels)
 };
+
+// The control block of a chain: uint64 wait limit, int status (+ 4 unused
+// bytes), kNumScalars doubles, and from kSlotOffset on one slot per CTA of a
+// global-memory team: two teams (all CTAs; the CTAs of the FP32 iterations) x
+// two buffers x four values of two tagged words.  Status, outputs and the
+// slots in use lie together, so one memset clears them before a launch.
+constexpr int kMaxTeam = 1024;
+constexpr int kNumScalars = 16;
+constexpr int kSlotWords = 32;              // 64-bit words per CTA
+constexpr int kTeamWords = kSlotWords / 2;  // ... of which per team
+constexpr size_t kSlotOffset = 256;
+constexpr size_t kControlBytes = kSlotOffset + (size_t)kMaxTeam * kSlotWords * 8;
+static_assert(16 + kNumScalars * 8 <= kSlotOffset, "control block header");
+
+inline void control_bind(ChainView* v, void* base) {
+    unsigned char* b = static_cast<unsigned char*>(base);
+    v->status = reinterpret_cast<int*>(b + 8);
+    v->scalars = reinterpret_cast<double*>(b + 16);
+    v->slots = reinterpret_cast<uint64_t*>(b + kSlotOffset);
+}
+
+// Clear status, outputs and the slots of a team of `team` CTAs.
+inline bool control_reset(const ChainView& v, int team, cudaStream_t s) {
+    const int ranks = team + v.team_pad < kMaxTeam ? team + v.team_pad : kMaxTeam;
+    return cudaMemsetAsync(v.status, 0,
+                           kSlotOffset - 8 + (size_t)ranks * kSlotWords * sizeof(uint64_t), s) ==
+           cudaSuccess;
+}
 
 }  // namespace hmc
 

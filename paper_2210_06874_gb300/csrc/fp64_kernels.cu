@@ -3,6 +3,7 @@
 //  k_cis        exp(i phi) table (one pass over phi)
 //  k_apply      one application of M or M^dag (one tile per CTA)
 //  k_force      F = phi/(delta U) + 2 Im(x conj(M^dag x))
+//               (both: dense tiles, or one slice per block by the series)
 //  k_cg         persistent CG solve of (M M^dag) x = chi
 //  k_trajectory persistent HMC trajectory: heat bath, leapfrog, Metropolis
 #include "fp64_path.cuh"
@@ -20,13 +21,13 @@ __global__ void k_cis(const double* __restrict__ phi, double2* __restrict__ cis,
 }
 
 template <bool DAG>
-__global__ void __launch_bounds__(NTHR) k_apply(ChainView c, const double2* in, double2* out) {
+__global__ void __launch_bounds__(NTHR) k_apply(const __grid_constant__ ChainView c, const double2* in, double2* out) {
     __shared__ Smem sm;
     EpiArgs ea = {};
     apply_tile<DAG, EPI_STORE>(c, blockIdx.x, in, out, ea, sm);
 }
 
-__global__ void __launch_bounds__(NTHR) k_force(ChainView c, const double* phi,
+__global__ void __launch_bounds__(NTHR) k_force(const __grid_constant__ ChainView c, const double* phi,
                                                 const double2* x, double* F) {
     __shared__ Smem sm;
     EpiArgs ea = {};
@@ -36,13 +37,36 @@ __global__ void __launch_bounds__(NTHR) k_force(ChainView c, const double* phi,
     apply_tile<true, EPI_FORCE>(c, blockIdx.x, x, nullptr, ea, sm);
 }
 
+// The same two by the series, one slice per block (its threads: the slice's
+// cells), with e^{i phi} computed in the tile: one launch, phi read once.
+template <bool DAG>
+__global__ void __launch_bounds__(NTHR) k_apply_series(const __grid_constant__ ChainView c, const double* phi,
+                                                       const double2* in, double2* out) {
+    extern __shared__ __align__(16) double hop_buf[];
+    EpiArgs ea = {};
+    ea.phi = phi;
+    series_tile<DAG, EPI_STORE, true>(c, blockIdx.x, 1, in, out, ea, hop_buf);
+}
+
+__global__ void __launch_bounds__(NTHR) k_force_series(const __grid_constant__ ChainView c, const double* phi,
+                                                       const double2* x, double* F) {
+    extern __shared__ __align__(16) double hop_buf[];
+    EpiArgs ea = {};
+    ea.phi = phi;
+    ea.F = F;
+    ea.inv_dU = 1.0 / (c.delta * c.U);
+    series_tile<true, EPI_FORCE, true>(c, blockIdx.x, 1, x, nullptr, ea, hop_buf);
+}
+
 __device__ __forceinline__ Team make_team(const ChainView& c) {
+    __shared__ unsigned s_gen;
+    if (threadIdx.x == 0) s_gen = 0;
     Team tm;
     tm.rank = blockIdx.x;
     tm.size = gridDim.x + c.team_pad;
-    tm.bar = c.bar;
     tm.status = c.status;
-    tm.partials = c.partials;
+    tm.slots = c.slots;
+    tm.gen = &s_gen;
     tm.cs = nullptr;
     return tm;
 }
@@ -78,14 +102,15 @@ __global__ void k_sum_partials(const double* __restrict__ partials, int n, doubl
 }
 
 // scalars: [0] iterations [1] true residual [2] status
-__global__ void __launch_bounds__(NTHR) k_cg(ChainView c, const double* phi, const double2* chi,
+template <int FORM>
+__global__ void __launch_bounds__(NTHR) k_cg(const __grid_constant__ ChainView c, const double* phi, const double2* chi,
                                              double2* x, double tol, int max_iter) {
     __shared__ Smem sm;
     Team tm = make_team(c);
     fill_cis(c, tm, phi);
     if (!team_barrier(tm)) return;
     CgResult res;
-    if (!cg_solve(c, tm, chi, x, tol, max_iter, res, sm)) return;
+    if (!cg_solve<FORM>(c, tm, chi, x, tol, max_iter, res, sm)) return;
     if (tm.rank == 0 && threadIdx.x == 0) {
         c.scalars[0] = res.iterations;
         c.scalars[1] = res.true_res;
@@ -94,7 +119,8 @@ __global__ void __launch_bounds__(NTHR) k_cg(ChainView c, const double* phi, con
 }
 
 // scalars: see TrajSlot in launch.h
-__global__ void __launch_bounds__(NTHR) k_trajectory(ChainView c, TrajArgs a) {
+template <int FORM>
+__global__ void __launch_bounds__(NTHR) k_trajectory(const __grid_constant__ ChainView c, TrajArgs a) {
     __shared__ Smem sm;
     Team tm = make_team(c);
     double* phi = a.phi;
@@ -122,7 +148,7 @@ __global__ void __launch_bounds__(NTHR) k_trajectory(ChainView c, TrajArgs a) {
     const double H0 = 0.5 * h0[0] * inv_dU + h0[1] + 0.5 * h0[2];
     // 2. chi = M rho
     EpiArgs ea = {};
-    apply_team<false, EPI_STORE>(c, tm, c.rho, c.chi, ea, sm);
+    apply_team<FORM, false, EPI_STORE>(c, tm, c.rho, c.chi, ea, sm);
     if (!team_barrier(tm)) return;
     // 3. leapfrog
     int iters = 0, solves = 0, status = HMC_OK;
@@ -145,13 +171,13 @@ __global__ void __launch_bounds__(NTHR) k_trajectory(ChainView c, TrajArgs a) {
             if (!team_barrier(tm)) return;
         }
         CgResult res;
-        if (!cg_solve(c, tm, c.chi, c.x, a.tol, a.max_iter, res, sm)) return;
+        if (!cg_solve<FORM>(c, tm, c.chi, c.x, a.tol, a.max_iter, res, sm)) return;
         iters += res.iterations;
         ++solves;
         max_res = fmax(max_res, res.true_res);
         if (res.status != HMC_OK && status == HMC_OK) status = res.status;
         ea.kick = md_kick(a, step) * ed;
-        apply_team<true, EPI_FORCE>(c, tm, c.x, nullptr, ea, sm);
+        apply_team<FORM, true, EPI_FORCE>(c, tm, c.x, nullptr, ea, sm);
         if (!team_barrier(tm)) return;
     }
     // 4. end energy and Metropolis
@@ -198,7 +224,8 @@ __global__ void __launch_bounds__(NTHR) k_trajectory(ChainView c, TrajArgs a) {
 //     F_B + F_1 = phi / (delta U) + 2 Im(x_1 conj(M_g^dag x_1)).
 // Consecutive inner kicks are merged.  Every solve starts from zero.
 // Scalars as k_trajectory, plus the outer level's CG iterations and solves.
-__global__ void __launch_bounds__(NTHR) k_trajectory_hb(ChainView c, TrajArgs a) {
+template <int FORM>
+__global__ void __launch_bounds__(NTHR) k_trajectory_hb(const __grid_constant__ ChainView c, TrajArgs a) {
     __shared__ Smem sm;
     Team tm = make_team(c);
     double* phi = a.phi;
@@ -232,18 +259,18 @@ __global__ void __launch_bounds__(NTHR) k_trajectory_hb(ChainView c, TrajArgs a)
     EpiArgs eg = {};
     eg.hop_m1 = gm1;
     EpiArgs e1 = {};
-    apply_team<false, EPI_STORE>(c, tm, c.rho, c.chi, eg, sm);
-    apply_team<false, EPI_STORE>(c, tm, c.xh, c.phi2, e1, sm);
+    apply_team<FORM, false, EPI_STORE>(c, tm, c.rho, c.chi, eg, sm);
+    apply_team<FORM, false, EPI_STORE>(c, tm, c.xh, c.phi2, e1, sm);
     if (!team_barrier(tm)) return;
     int iters_in = 0, iters_out = 0, solves_in = 0, solves_out = 0, status = HMC_OK;
     double max_res = 0.0;
     CgResult res;
-    if (!cg_solve(c, tm, c.phi2, c.x2, a.tol, a.max_iter, res, sm, false, gm1)) return;
+    if (!cg_solve<FORM>(c, tm, c.phi2, c.x2, a.tol, a.max_iter, res, sm, false, gm1)) return;
     iters_in += res.iterations;
     ++solves_in;
     max_res = fmax(max_res, res.true_res);
     if (res.status != HMC_OK) status = res.status;
-    apply_team<true, EPI_STORE>(c, tm, c.x2, c.chi2, eg, sm);
+    apply_team<FORM, true, EPI_STORE>(c, tm, c.x2, c.chi2, eg, sm);
     if (!team_barrier(tm)) return;
     // 3. nested leapfrog
     const double ed = a.eps * c.delta;
@@ -260,7 +287,7 @@ __global__ void __launch_bounds__(NTHR) k_trajectory_hb(ChainView c, TrajArgs a)
     };
     auto kick_inner = [&](double cf) {
         CgResult r;
-        if (!cg_solve(c, tm, c.chi, c.x, a.tol, a.max_iter, r, sm, false, gm1)) return false;
+        if (!cg_solve<FORM>(c, tm, c.chi, c.x, a.tol, a.max_iter, r, sm, false, gm1)) return false;
         iters_in += r.iterations;
         ++solves_in;
         max_res = fmax(max_res, r.true_res);
@@ -271,14 +298,14 @@ __global__ void __launch_bounds__(NTHR) k_trajectory_hb(ChainView c, TrajArgs a)
         ef.pi = c.pi;
         ef.inv_dU = inv_dU;
         ef.kick = cf * ed;
-        apply_team<true, EPI_FORCE>(c, tm, c.x, nullptr, ef, sm);
+        apply_team<FORM, true, EPI_FORCE>(c, tm, c.x, nullptr, ef, sm);
         return team_barrier(tm);
     };
     auto kick_outer = [&](double cf) {
-        apply_team<false, EPI_STORE>(c, tm, c.chi2, c.phi2, eg, sm);   // phi_2 = M_g chi_2
+        apply_team<FORM, false, EPI_STORE>(c, tm, c.chi2, c.phi2, eg, sm);   // phi_2 = M_g chi_2
         if (!team_barrier(tm)) return false;
         CgResult r;
-        if (!cg_solve(c, tm, c.phi2, c.x2, a.tol, a.max_iter, r, sm)) return false;
+        if (!cg_solve<FORM>(c, tm, c.phi2, c.x2, a.tol, a.max_iter, r, sm)) return false;
         iters_out += r.iterations;
         ++solves_out;
         max_res = fmax(max_res, r.true_res);
@@ -288,11 +315,11 @@ __global__ void __launch_bounds__(NTHR) k_trajectory_hb(ChainView c, TrajArgs a)
         ef.pi = c.pi;
         ef.inv_dU = 0.0;              // the bosonic force sits on the inner level
         ef.kick = cf * ed;
-        apply_team<true, EPI_FORCE>(c, tm, c.x2, nullptr, ef, sm);
+        apply_team<FORM, true, EPI_FORCE>(c, tm, c.x2, nullptr, ef, sm);
         if (!team_barrier(tm)) return false;
         ef.hop_m1 = gm1;
         ef.chi = c.chi2;
-        apply_team<true, EPI_RATIO>(c, tm, c.x2, nullptr, ef, sm);
+        apply_team<FORM, true, EPI_RATIO>(c, tm, c.x2, nullptr, ef, sm);
         return team_barrier(tm);
     };
     if (!kick_outer(0.5)) return;
@@ -358,59 +385,96 @@ static cudaError_t launch_coop(const void* kernel, int grid, int threads, void**
     return cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args, 0, s);
 }
 
-int launch_cis_f64(const ChainView& c, const double* phi, cudaStream_t s) {
+static int launch_cis_f64(const ChainView& c, const double* phi, cudaStream_t s) {
     int blocks = (c.N + 255) / 256;
     if (blocks > 4096) blocks = 4096;
     f64::k_cis<<<blocks, 256, 0, s>>>(phi, c.cis, c.N);
     return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
 }
 
-int launch_apply_f64(const ChainView& c, bool dag, const double2* in, double2* out,
-                     cudaStream_t s) {
-    const int nt = ((c.V + f64::TI - 1) / f64::TI) * ((c.Nt + f64::TT - 1) / f64::TT);
+static int dense_tiles(const ChainView& c) {
+    return ((c.V + f64::TI - 1) / f64::TI) * ((c.Nt + f64::TT - 1) / f64::TT);
+}
+
+// Threads of a one-slice series block: a warp multiple covering the cells.
+static int series_threads(const ChainView& c) {
+    const int t = (c.V / 2 + 31) / 32 * 32;
+    return t < f64::NTHR ? t : f64::NTHR;
+}
+
+int launch_apply_f64(const ChainView& c, bool dag, const double* phi, const double2* in,
+                     double2* out, cudaStream_t s) {
+    if (f64::series_form(c, c.V)) {
+        const int thr = series_threads(c);
+        const size_t sm = (size_t)c.V * sizeof(double);
+        if (dag)
+            f64::k_apply_series<true><<<c.Nt, thr, sm, s>>>(c, phi, in, out);
+        else
+            f64::k_apply_series<false><<<c.Nt, thr, sm, s>>>(c, phi, in, out);
+        return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
+    }
+    const int st = launch_cis_f64(c, phi, s);
+    if (st != HMC_OK) return st;
     if (dag)
-        f64::k_apply<true><<<nt, f64::NTHR, 0, s>>>(c, in, out);
+        f64::k_apply<true><<<dense_tiles(c), f64::NTHR, 0, s>>>(c, in, out);
     else
-        f64::k_apply<false><<<nt, f64::NTHR, 0, s>>>(c, in, out);
+        f64::k_apply<false><<<dense_tiles(c), f64::NTHR, 0, s>>>(c, in, out);
     return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
 }
 
 int launch_force_f64(const ChainView& c, const double* phi, const double2* x, double* F,
                      cudaStream_t s) {
-    const int nt = ((c.V + f64::TI - 1) / f64::TI) * ((c.Nt + f64::TT - 1) / f64::TT);
-    f64::k_force<<<nt, f64::NTHR, 0, s>>>(c, phi, x, F);
+    if (f64::series_form(c, c.V)) {
+        f64::k_force_series<<<c.Nt, series_threads(c), (size_t)c.V * sizeof(double), s>>>(
+            c, phi, x, F);
+        return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
+    }
+    const int st = launch_cis_f64(c, phi, s);
+    if (st != HMC_OK) return st;
+    f64::k_force<<<dense_tiles(c), f64::NTHR, 0, s>>>(c, phi, x, F);
     return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
+}
+
+// CTAs worth launching for the tiles of one application.
+static int f64_tiles(const ChainView& c) {
+    return f64::series_form(c, f64::kHopDoubles) ? c.Nt : dense_tiles(c);
 }
 
 int launch_action(const ChainView& c, const double* phi, const double2* chi, const double2* x,
                   double* out, cudaStream_t s) {
     int blocks = (c.N + 255) / 256;
     if (blocks > 1024) blocks = 1024;
+    double* partials = reinterpret_cast<double*>(c.slots);   // free between launches
     f64::k_action_partials<<<blocks, 256, 0, s>>>(phi, chi, x, c.N, 0.5 / (c.delta * c.U),
-                                                 c.partials);
-    f64::k_sum_partials<<<1, 256, 0, s>>>(c.partials, blocks, out);
+                                                 partials);
+    f64::k_sum_partials<<<1, 256, 0, s>>>(partials, blocks, out);
     return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
 }
 
 int launch_cg_f64(const ChainView& c, int num_sms, const double* phi, const double2* chi,
                   double2* x, double tol, int max_iter, cudaStream_t s) {
-    const int nt = ((c.V + f64::TI - 1) / f64::TI) * ((c.Nt + f64::TT - 1) / f64::TT);
-    const int grid = persistent_grid((const void*)f64::k_cg, f64::NTHR, num_sms, nt);
-    if (grid < 1) return HMC_ERR_CUDA;
+    const void* fn = f64::series_form(c, f64::kHopDoubles)
+                         ? (const void*)f64::k_cg<f64::FORM_SERIES>
+                         : (const void*)f64::k_cg<f64::FORM_DENSE>;
+    const int grid = persistent_grid(fn, f64::NTHR, num_sms, f64_tiles(c));
+    if (grid < 1 || !control_reset(c, grid, s)) return HMC_ERR_CUDA;
     ChainView cv = c;
     void* args[] = {&cv, &phi, &chi, &x, &tol, &max_iter};
-    return launch_coop((const void*)f64::k_cg, grid, f64::NTHR, args, s) == cudaSuccess
+    return launch_coop(fn, grid, f64::NTHR, args, s) == cudaSuccess
                ? HMC_OK
                : HMC_ERR_CUDA;
 }
 
 int launch_trajectory_f64(const ChainView& c, int num_sms, const TrajArgs& a, cudaStream_t s) {
-    const int nt = ((c.V + f64::TI - 1) / f64::TI) * ((c.Nt + f64::TT - 1) / f64::TT);
-    const void* fn = a.hb_inner > 0 ? (const void*)f64::k_trajectory_hb
-                                    : (const void*)f64::k_trajectory;
+    const bool ser = f64::series_form(c, f64::kHopDoubles);
+    const void* fn = a.hb_inner > 0
+                         ? (ser ? (const void*)f64::k_trajectory_hb<f64::FORM_SERIES>
+                                : (const void*)f64::k_trajectory_hb<f64::FORM_DENSE>)
+                         : (ser ? (const void*)f64::k_trajectory<f64::FORM_SERIES>
+                                : (const void*)f64::k_trajectory<f64::FORM_DENSE>);
     if (a.hb_inner > 0 && (!c.chi2 || !c.phi2 || !c.x2)) return HMC_ERR_BAD_ARG;
-    const int grid = persistent_grid(fn, f64::NTHR, num_sms, nt);
-    if (grid < 1) return HMC_ERR_CUDA;
+    const int grid = persistent_grid(fn, f64::NTHR, num_sms, f64_tiles(c));
+    if (grid < 1 || !control_reset(c, grid, s)) return HMC_ERR_CUDA;
     ChainView cv = c;
     TrajArgs av = a;
     void* args[] = {&cv, &av};

@@ -51,12 +51,12 @@ enum TrajSlot : int {
     kTrajDH = 0, kTrajH0, kTrajH1, kTrajU, kTrajAccept, kTrajIters, kTrajSolves,
     kTrajRU, kTrajMaxRes, kTrajStatus, kTrajFp64Iters, kTrajItersOuter,
     // 12 and 13 keep the mixed CG's segment state
-    kTrajSolvesOuter = 14, kNumScalars = 16
+    kTrajSolvesOuter = 14
 };
+static_assert(kTrajSolvesOuter < kNumScalars, "scalar slots");
 
-int launch_cis_f64(const ChainView& c, const double* phi, cudaStream_t s);
-int launch_apply_f64(const ChainView& c, bool dag, const double2* in, double2* out,
-                     cudaStream_t s);
+int launch_apply_f64(const ChainView& c, bool dag, const double* phi, const double2* in,
+                     double2* out, cudaStream_t s);
 int launch_force_f64(const ChainView& c, const double* phi, const double2* x, double* F,
                      cudaStream_t s);
 int launch_action(const ChainView& c, const double* phi, const double2* chi, const double2* x,

@@ -7,8 +7,8 @@
 // from growing the device heap.  They cannot create an hmc_ctx, whose
 // workspaces are cudaMalloc'ed.  This entry point runs the same persistent
 // FP64 CG kernel as hmc_cg_solve(prec = HMC_PREC_FP64), but its scratch (the
-// exp(i phi) table, the CG vectors r, p, q, the team partial sums, the
-// barrier and status words) lives in one file-scope __device__ array that
+// exp(i phi) table, the CG vectors r, p (twice), q, the status word and the team's
+// partial sums) lives in one file-scope __device__ array that
 // every GPU loading the library holds until exit.  The call waits for its
 // own result (it copies the statistics to the host and synchronises the
 // stream), so it refuses to run on a stream that is being captured into a
@@ -28,16 +28,13 @@ namespace {
 // Largest space-time volume N = V * Nt the static scratch holds.
 constexpr int kNoAllocMaxN = 32768;
 constexpr size_t kVecBytes = sizeof(double2) * (size_t)kNoAllocMaxN;
-constexpr size_t kPartialBytes = sizeof(double) * kPartialDoubles;
-// layout: cis | r | p | q | partials | scalars[16] | bar[2] | status
+// layout: cis | r | p | q | p2 | control block (never written: its wait limit)
 constexpr size_t kOffR = kVecBytes;
 constexpr size_t kOffP = 2 * kVecBytes;
 constexpr size_t kOffQ = 3 * kVecBytes;
-constexpr size_t kOffPartials = 4 * kVecBytes;
-constexpr size_t kOffScalars = kOffPartials + kPartialBytes;
-constexpr size_t kOffBar = kOffScalars + 16 * sizeof(double);
-constexpr size_t kOffStatus = kOffBar + 256;
-constexpr size_t kScratchBytes = kOffStatus + 256;  // about 2.1 MB
+constexpr size_t kOffP2 = 4 * kVecBytes;
+constexpr size_t kOffControl = 5 * kVecBytes;
+constexpr size_t kScratchBytes = kOffControl + kControlBytes;  // about 2.9 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -133,13 +130,8 @@ extern "C" int hmc_cg_solve_noalloc(const double* E, int L, int Nt, const double
     v.r = reinterpret_cast<double2*>(b + kOffR);
     v.p = reinterpret_cast<double2*>(b + kOffP);
     v.q = reinterpret_cast<double2*>(b + kOffQ);
-    v.partials = reinterpret_cast<double*>(b + kOffPartials);
-    v.scalars = reinterpret_cast<double*>(b + kOffScalars);
-    v.bar = reinterpret_cast<unsigned*>(b + kOffBar);
-    v.status = reinterpret_cast<int*>(b + kOffStatus);
-    // the barrier must start at zero, the status word and the outputs clear
-    if (cudaMemsetAsync(b + kOffScalars, 0, kScratchBytes - kOffScalars, s) != cudaSuccess)
-        return HMC_ERR_CUDA;
+    v.p2 = reinterpret_cast<double2*>(b + kOffP2);
+    control_bind(&v, b + kOffControl);
     st = launch_cg_f64(v, num_sms, phi, (const double2*)chi, (double2*)x, tol, max_iter, s);
     if (st != HMC_OK) return st;
     double out[3];

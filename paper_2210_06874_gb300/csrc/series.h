@@ -1,0 +1,91 @@
+// series.h -- E = exp(delta (kappa h - mu)) as a polynomial of the sparse
+// hopping h (host part; the device functions are in fp64_path.cuh and
+// series_cg.cuh).
+//
+// h has three neighbours per site and its eigenvalues lie in [-3, 3], so with
+// rho = 3 |delta kappa| a polynomial of degree K reaches a given accuracy once
+// the Chebyshev tail 2 (rho / 2)^(K+1) / (K+1)! is below it: K = 11 for FP64
+// and 6 for FP32 at delta kappa = 1/8, on every lattice size, against V
+// multiply-adds per site for the dense product.  Horner's form
+//     E v = c0 y_1,  y_{K+1} = v,  y_k = v + ratio_k h y_{k+1}
+// costs two additions and one multiply-add per site, component and degree.
+#pragma once
+
+#include <math.h>
+
+namespace hmc {
+
+constexpr int kSerMax64 = 40;   // largest degree kept (FP64)
+constexpr int kSerMax32 = 24;   // largest degree kept (FP32)
+
+struct HopSeries {
+    int ok;                     // the series may be used (0: the dense E only)
+    int k64, k32;               // degrees
+    double c0;                  // FP64 polynomial's constant, includes e^{-delta mu}
+    float c0f;                  // FP32 polynomial's constant, likewise
+    double r64[kSerMax64];      // r64[k-1] = c_k / c_{k-1}
+    float r32[kSerMax32];
+};
+
+// Largest rho the series is used for (beyond it the degree and the growth
+// e^rho of the terms make the dense product the better choice), and the
+// largest L (4 cells per thread of a 256-thread block).
+constexpr double kSerMaxRho = 4.0;
+constexpr int kSerMaxL = 32;
+
+// Economised power series of exp(rho t) on |t| <= 1: from the Taylor
+// coefficients rho^m / m!, each power t^m above the degree is replaced by its
+// best lower-degree approximation t^m - 2^{1-m} T_m(t), highest first, which
+// costs 2^{1-m} times its coefficient.  Returns the smallest degree <= most
+// whose dropped terms stay below tol (-1: none), coefficients in b.
+inline int series_degree(double rho, double tol, int most, double* b) {
+    constexpr int M = 96;       // rho <= 4: rho^96 / 96! < 1e-91
+    double a[M + 1];
+    a[0] = 1.0;
+    for (int m = 1; m <= M; ++m) a[m] = a[m - 1] * rho / m;
+    double err = 0.0;
+    int K = M;
+    while (K > 0) {
+        const double cost = ldexp(fabs(a[K]), 1 - K);
+        if (err + cost > tol) break;
+        err += cost;
+        // t^K = 2^{1-K} T_K - sum_{j>=1} 2^{1-K} tc_j t^{K-2j}, with the
+        // coefficient of t^{K-2j} in T_K:
+        //   tc_j = (-1)^j (K/2) (K-j-1)! / (j! (K-2j)!) 2^{K-2j}
+        // (ratio of consecutive ones below)
+        double tc = ldexp(1.0, K - 1);
+        for (int j = 1; 2 * j <= K; ++j) {
+            tc *= -(double)(K - 2 * j + 2) * (K - 2 * j + 1) / (4.0 * j * (K - j));
+            a[K - 2 * j] -= a[K] * ldexp(tc, 1 - K);
+        }
+        --K;
+    }
+    if (K > most) return -1;
+    for (int m = 0; m <= K; ++m) b[m] = a[m];
+    return K;
+}
+
+// Series of exp(dk h) times f on an L x L lattice.
+inline void hop_series_build(int L, double dk, double f, HopSeries* s) {
+    *s = HopSeries{};
+    s->c0 = f;
+    const double rho = 3.0 * fabs(dk);
+    if (!(rho <= kSerMaxRho) || L > kSerMaxL) return;
+    double b[97];
+    // tolerances relative to the smallest singular value e^{-rho} of E: a
+    // tenth of a rounding of the result in each precision
+    const int k64 = series_degree(rho, 2e-17 * exp(-rho), kSerMax64, b);
+    if (k64 < 0) return;
+    const double sg = dk < 0.0 ? -1.0 : 1.0;
+    s->c0 = f * b[0];
+    for (int k = 1; k <= k64; ++k) s->r64[k - 1] = sg * b[k] / b[k - 1] / 3.0;
+    const int k32 = series_degree(rho, 6e-9 * exp(-rho), kSerMax32, b);
+    if (k32 < 0) return;
+    s->c0f = (float)(f * b[0]);
+    for (int k = 1; k <= k32; ++k) s->r32[k - 1] = (float)(sg * b[k] / b[k - 1] / 3.0);
+    s->k64 = k64;
+    s->k32 = k32;
+    s->ok = 1;
+}
+
+}  // namespace hmc

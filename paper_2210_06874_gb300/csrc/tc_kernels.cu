@@ -390,7 +390,7 @@ template <bool DAG>
 __global__ void __launch_bounds__(NTHR, 1)
     k_apply(const __grid_constant__ CUtensorMap mhi, const __grid_constant__ CUtensorMap mlo,
             const __grid_constant__ CUtensorMap bhi, const __grid_constant__ CUtensorMap blo,
-            ChainView c, int ns_tile, const float2* in, float2* out, const float* inv) {
+            const __grid_constant__ ChainView c, int ns_tile, const float2* in, float2* out, const float* inv) {
     extern __shared__ __align__(1024) uint8_t dyn[];
     TcState st;
     tc_setup(st, dyn, c.status);
@@ -418,7 +418,7 @@ template <bool DAG>
 __global__ void __launch_bounds__(NTHR, 1)
     k_apply_w(const __grid_constant__ CUtensorMap mhi, const __grid_constant__ CUtensorMap mlo,
               const __grid_constant__ CUtensorMap uhi, const __grid_constant__ CUtensorMap ulo,
-              ChainView c, int W, int ns_tile, int csplit, const float2* in, float2* out,
+              const __grid_constant__ ChainView c, int W, int ns_tile, int csplit, const float2* in, float2* out,
               const float* inv) {
     extern __shared__ __align__(1024) uint8_t dyn[];
     TcState st;
@@ -511,7 +511,7 @@ template <bool DAG>
 __global__ void __launch_bounds__(NTHR, 1)
     k_apply_sk(const __grid_constant__ CUtensorMap mhi, const __grid_constant__ CUtensorMap mlo,
                const __grid_constant__ CUtensorMap bhi, const __grid_constant__ CUtensorMap blo,
-               ChainView c, int C, int ns, const float2* in, float2* out, const float* inv) {
+               const __grid_constant__ ChainView c, int C, int ns, const float2* in, float2* out, const float* inv) {
     extern __shared__ __align__(1024) uint8_t dyn[];
     TcState st;
     tc_setup(st, dyn, c.status);
@@ -593,16 +593,27 @@ struct BatchCallArgs {
     double* phi;               // packed fields of all chains
 };
 
+// Form of E in the FP64 steps of a kernel of kind KIND: the tensor-core tiles
+// whose FP32 loop is inlined keep the dense form, because a kernel with the
+// series in it gives that loop fewer registers (10-20 % of its time); the
+// split-K loop is a function of its own and takes the series where it exists.
+// Kernel kinds of the FP32 iterations: site-major tensor-core tiles, the
+// CUDA-core cluster solver, slice-major and split-K tensor-core tiles.
+enum TileKind : int { kKindSite = 0, kKindSmall = 1, kKindSlice = 2, kKindSplitK = 3 };
+template <int KIND>
+constexpr int kForm = KIND == kKindSplitK ? f64::FORM_EITHER : f64::FORM_DENSE;
+
 // FP64 true residual of x64: r64 = chi - M (M^dag x64); returns |r64|^2.
+template <int FORM>
 __device__ bool f64_residual(const ChainView& c, Team& tm, f64::Smem& sm, const double2* chi,
                              double2* x64, double& rr, double gm1 = 0.0) {
     f64::EpiArgs ea = {};
     ea.hop_m1 = gm1;   // M_g = 1 - g S E D with g = 1 + gm1 (mass preconditioning)
-    f64::apply_team<true, f64::EPI_STORE>(c, tm, x64, c.q, ea, sm);
+    f64::apply_team<FORM, true, f64::EPI_STORE>(c, tm, x64, c.q, ea, sm);
     if (!team_barrier(tm)) return false;
     ea.chi = chi;
     ea.r = c.r;
-    double v[1] = {f64::apply_team<false, f64::EPI_RESIDUAL>(c, tm, c.q, nullptr, ea, sm)};
+    double v[1] = {f64::apply_team<FORM, false, f64::EPI_RESIDUAL>(c, tm, c.q, nullptr, ea, sm)};
     if (!team_sum<1>(tm, v)) return false;
     rr = v[0];
     return true;
@@ -861,10 +872,6 @@ __device__ __noinline__ int sk_segment(const ChainView& c, Team& ti, TcState& st
     return reason;
 }
 
-// Kernel kinds of the FP32 iterations: site-major tensor-core tiles, the
-// CUDA-core cluster solver, slice-major tensor-core tiles.
-enum TileKind : int { kKindSite = 0, kKindSmall = 1, kKindSlice = 2, kKindSplitK = 3 };
-
 template <int KIND>
 __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& sm64,
                          const CUtensorMap* mhi, const CUtensorMap* mlo,
@@ -882,7 +889,8 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
     const bool in_inner = tm.rank < inner_size;
     Team ti = tm;
     ti.size = inner_size;
-    ti.bar = c.bar + 2;
+    ti.slots = tm.slots + kTeamWords;
+    ti.gen = tm.gen + 1;
     // inner team = cluster 0: its barriers stay inside the cluster
     ti.cs = (ics && pa.cluster > 1 && inner_size == pa.cluster) ? ics : nullptr;
     // FP64 solution and |chi|^2 on all CTAs
@@ -909,7 +917,7 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
     double rr_true = chi2;
     const double2* r0 = chi;
     if (warm) {
-        if (!f64_residual(c, tm, sm64, chi, x64, rr_true, gm1)) return false;
+        if (!f64_residual<kForm<KIND>>(c, tm, sm64, chi, x64, rr_true, gm1)) return false;
         ++res.reliable_updates;
         if (!finite_d(rr_true)) {
             res.status = HMC_ERR_NONFINITE;
@@ -1131,7 +1139,7 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
         const int it = (int)seg[1];
         if (reason == kSegNonfinite) { res.status = HMC_ERR_NONFINITE; break; }
         // FP64 true residual on all CTAs
-        if (!f64_residual(c, tm, sm64, chi, x64, rr_true, gm1)) return false;
+        if (!f64_residual<kForm<KIND>>(c, tm, sm64, chi, x64, rr_true, gm1)) return false;
         ++res.reliable_updates;
         if (!finite_d(rr_true)) { res.status = HMC_ERR_NONFINITE; break; }
         if (rr_true <= stop) { conv = true; break; }
@@ -1159,8 +1167,9 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
         // FP64 CG on all CTAs from the current solution; its final true
         // residual leaves M^dag x in q, as the reliable update does
         f64::CgResult r64;
-        if (!f64::cg_solve(c, tm, chi, x64, pa.tol, max(1, pa.max_iter - res.iterations), r64,
-                           sm64, true, gm1))
+        if (!f64::cg_solve<kForm<KIND>>(c, tm, chi, x64, pa.tol,
+                                        max(1, pa.max_iter - res.iterations), r64, sm64, true,
+                                        gm1))
             return false;
         res.fp64_iterations = r64.iterations;
         res.true_res = r64.true_res;
@@ -1183,12 +1192,14 @@ __device__ inline void cluster_begin(const PersistentArgs& pa, ClusterSync* cs, 
 }
 
 __device__ __forceinline__ Team make_team(const ChainView& c) {
+    __shared__ unsigned s_gen[2];   // syncs of the whole team and of the inner one
+    if (threadIdx.x == 0) s_gen[0] = s_gen[1] = 0;
     Team tm;
     tm.rank = blockIdx.x;
     tm.size = gridDim.x + c.team_pad;
-    tm.bar = c.bar;
     tm.status = c.status;
-    tm.partials = c.partials;
+    tm.slots = c.slots;
+    tm.gen = s_gen;
     tm.cs = nullptr;
     return tm;
 }
@@ -1225,7 +1236,7 @@ __device__ inline void persistent_teardown(TcState& st) {
 template <int KIND>
 __global__ void __launch_bounds__(NTHR, 1)
     k_cg(const __grid_constant__ CUtensorMap mhi, const __grid_constant__ CUtensorMap mlo,
-         ChainView c, PersistentArgs pa, const double* phi, const double2* chi, double2* x) {
+         const __grid_constant__ ChainView c, PersistentArgs pa, const double* phi, const double2* chi, double2* x) {
     extern __shared__ __align__(1024) uint8_t dyn[];
     __shared__ f64::Smem sm64;
     TcState st;
@@ -1278,7 +1289,7 @@ __device__ bool run_trajectory(const ChainView& c, Team& tm, TcState& st, f64::S
     const double H0 = 0.5 * h0[0] * inv_dU + h0[1] + 0.5 * h0[2];
     f64::EpiArgs ea = {};
     if (ok) {
-        f64::apply_team<false, f64::EPI_STORE>(c, tm, c.rho, c.chi, ea, sm64);
+        f64::apply_team<kForm<KIND>, false, f64::EPI_STORE>(c, tm, c.rho, c.chi, ea, sm64);
         ok = team_barrier(tm);
     }
     int iters = 0, solves = 0, rus = 0, fp64_iters = 0, status = HMC_OK;
@@ -1338,7 +1349,7 @@ __device__ bool run_trajectory(const ChainView& c, Team& tm, TcState& st, f64::S
                 c.pi[e] -= ea.kick * f;
             }
         } else {
-            f64::apply_team<true, f64::EPI_FORCE>(c, tm, c.x, nullptr, ea, sm64);
+            f64::apply_team<kForm<KIND>, true, f64::EPI_FORCE>(c, tm, c.x, nullptr, ea, sm64);
         }
         ok = team_barrier(tm);
     }
@@ -1439,8 +1450,8 @@ __device__ __noinline__ bool run_trajectory_hb(const ChainView& c, Team& tm, TcS
     f64::EpiArgs eg = {};
     eg.hop_m1 = gm1;
     f64::EpiArgs e1 = {};
-    f64::apply_team<false, f64::EPI_STORE>(c, tm, c.rho, c.chi, eg, sm64);
-    f64::apply_team<false, f64::EPI_STORE>(c, tm, c.xh, c.phi2, e1, sm64);
+    f64::apply_team<kForm<KIND>, false, f64::EPI_STORE>(c, tm, c.rho, c.chi, eg, sm64);
+    f64::apply_team<kForm<KIND>, false, f64::EPI_STORE>(c, tm, c.xh, c.phi2, e1, sm64);
     if (!team_barrier(tm)) return false;
     MixedResult res{};
     if (!cg_mixed<KIND>(c, tm, st, sm64, mhi, mlo, pa, ics, c.phi2, c.x2, res, false, gm1))
@@ -1449,7 +1460,7 @@ __device__ __noinline__ bool run_trajectory_hb(const ChainView& c, Team& tm, TcS
     if (res.status == HMC_OK) {
         HMC_TEAM_ELEMS(e, c, tm) c.chi2[e] = c.q[e];   // q = M_g^dag x_2 (final residual)
     } else {
-        f64::apply_team<true, f64::EPI_STORE>(c, tm, c.x2, c.chi2, eg, sm64);
+        f64::apply_team<kForm<KIND>, true, f64::EPI_STORE>(c, tm, c.x2, c.chi2, eg, sm64);
     }
     if (!team_barrier(tm)) return false;
     // 3. nested leapfrog
@@ -1487,13 +1498,13 @@ __device__ __noinline__ bool run_trajectory_hb(const ChainView& c, Team& tm, TcS
             ef.pi = c.pi;
             ef.inv_dU = inv_dU;
             ef.kick = k;
-            f64::apply_team<true, f64::EPI_FORCE>(c, tm, c.x, nullptr, ef, sm64);
+            f64::apply_team<kForm<KIND>, true, f64::EPI_FORCE>(c, tm, c.x, nullptr, ef, sm64);
         }
         return team_barrier(tm);
     };
     // ratio force: F_2 = 2 Im(x_2 conj(M^dag x_2)) - 2 Im(conj(M_g^dag x_2 - x_2) chi_2)
     auto kick_outer = [&](double cf) {
-        f64::apply_team<false, f64::EPI_STORE>(c, tm, c.chi2, c.phi2, eg, sm64);   // M_g chi_2
+        f64::apply_team<kForm<KIND>, false, f64::EPI_STORE>(c, tm, c.chi2, c.phi2, eg, sm64);   // M_g chi_2
         if (!team_barrier(tm)) return false;
         MixedResult r{};
         if (!cg_mixed<KIND>(c, tm, st, sm64, mhi, mlo, pa, ics, c.phi2, c.x2, r, warm_out, 0.0))
@@ -1512,12 +1523,12 @@ __device__ __noinline__ bool run_trajectory_hb(const ChainView& c, Team& tm, TcS
                 c.pi[e] -= k * (2.0 * (xv.y * y.x - xv.x * y.y));
             }
         } else {
-            f64::apply_team<true, f64::EPI_FORCE>(c, tm, c.x2, nullptr, ef, sm64);
+            f64::apply_team<kForm<KIND>, true, f64::EPI_FORCE>(c, tm, c.x2, nullptr, ef, sm64);
         }
         if (!team_barrier(tm)) return false;
         ef.hop_m1 = gm1;
         ef.chi = c.chi2;
-        f64::apply_team<true, f64::EPI_RATIO>(c, tm, c.x2, nullptr, ef, sm64);
+        f64::apply_team<kForm<KIND>, true, f64::EPI_RATIO>(c, tm, c.x2, nullptr, ef, sm64);
         return team_barrier(tm);
     };
     if (!kick_outer(0.5)) return false;
@@ -1569,7 +1580,7 @@ __device__ __noinline__ bool run_trajectory_hb(const ChainView& c, Team& tm, TcS
 template <int KIND>
 __global__ void __launch_bounds__(NTHR, 1)
     k_trajectory(const __grid_constant__ CUtensorMap mhi,
-                 const __grid_constant__ CUtensorMap mlo, ChainView c, PersistentArgs pa,
+                 const __grid_constant__ CUtensorMap mlo, const __grid_constant__ ChainView c, PersistentArgs pa,
                  TrajArgs a) {
     extern __shared__ __align__(1024) uint8_t dyn[];
     __shared__ f64::Smem sm64;
@@ -1689,9 +1700,7 @@ __global__ void __launch_bounds__(NTHR, 1)
                 Team tm{};
                 tm.rank = 0;
                 tm.size = 1;
-                tm.bar = it.v.bar;
-                tm.status = it.v.status;
-                tm.partials = it.v.partials;
+                tm.status = it.v.status;   // one CTA or one cluster: no slots
                 tm.cs = nullptr;
                 batch_run(it, ci, call, outs, st, sm64, tm, nullptr, true, ok);
             }
@@ -1702,9 +1711,7 @@ __global__ void __launch_bounds__(NTHR, 1)
         Team tm{};
         tm.rank = crank;
         tm.size = csize;
-        tm.bar = it.v.bar;
-        tm.status = it.v.status;
-        tm.partials = it.v.partials;
+        tm.status = it.v.status;   // one CTA or one cluster: no slots
         tm.cs = &s_cs;
         batch_run(it, ci, call, outs, st, sm64, tm, &s_cs, crank == 0, ok);
         // the team's outcome, the same on every member: a failed member has
@@ -1727,9 +1734,7 @@ __global__ void __launch_bounds__(NTHR, 1)
         Team tm{};
         tm.rank = 0;
         tm.size = 1;
-        tm.bar = it.v.bar;
-        tm.status = it.v.status;
-        tm.partials = it.v.partials;
+        tm.status = it.v.status;   // one CTA or one cluster: no slots
         tm.cs = nullptr;
         batch_run(it, ci, call, outs, st, sm64, tm, nullptr, true, ok);
         // a failed bounded wait leaves the operand ring in an unknown phase:
@@ -2269,6 +2274,7 @@ static tc::PersistentArgs persistent_args(hmc_ctx* c, int grid, double tol, int 
 static int launch_persistent(hmc_ctx* c, const void* fn, int grid, void** args,
                              tc::PersistentArgs& pa, cudaStream_t s) {
     int cm = c->params.cluster_mode;
+    if (!control_reset(c->view, grid, s)) return HMC_ERR_CUDA;
     if (pa.mode == tc::kSmall) {
         // the small mode reads its peers' shared memory: a cluster or nothing
         if (pa.inner < 1 || grid % pa.inner != 0) return HMC_ERR_UNSUPPORTED;
@@ -2346,8 +2352,9 @@ static int launch_splitk(hmc_ctx* c, const void* fn, void** args, tc::Persistent
     // CTA runs; were one not resident, the bounded team waits would end the
     // launch with HMC_ERR_TIMEOUT.
     cfg.numAttrs = getenv("HMC_PROFILE_NONCOOPERATIVE") ? 1 : 2;
-    if (cudaMemsetAsync(c->view.gslots, 0, tc::kGatherSlots * sizeof(unsigned long long), s) !=
-        cudaSuccess)
+    if (!control_reset(c->view, grid, s) ||
+        cudaMemsetAsync(c->view.gslots, 0, tc::kGatherSlots * sizeof(unsigned long long), s) !=
+            cudaSuccess)
         return HMC_ERR_CUDA;
     pa.cluster = pa.sk_C;
     if (cudaLaunchKernelExC(&cfg, fn, args) != cudaSuccess) {
