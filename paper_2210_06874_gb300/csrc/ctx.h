@@ -53,6 +53,11 @@ struct ChainView {
     // rows, 128-byte swizzle); null when the context has no split-K shape
     const void* sk_maps;
     unsigned long long* gslots; // sequence-numbered partial sums and totals (tc_splitk.cuh)
+    // FP32 iterations by the series (series_cg.cuh): boundary slices and norms
+    // between the CTAs of a team, and the last sequence number used
+    uint64_t* ser_mail;         // [2][ser_ctas][V] x 2 words
+    uint64_t* ser_norm;         // [2][ser_ctas] every 16 words
+    unsigned* ser_seq;
     // control block (control_bind below): wait limit, status word, outputs of
     // the call, team slots
     int* status;

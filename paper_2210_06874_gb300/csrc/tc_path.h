@@ -16,6 +16,20 @@ int tc_cg(hmc_ctx* c, const double* phi, const double2* chi, double2* x, double 
           int max_iter, cudaStream_t s);
 int tc_trajectory(hmc_ctx* c, const TrajArgs& a, cudaStream_t s);
 
+// E by the series (series_kernels.cu): the automatic choice (operand_mode and
+// cluster_mode 0) where it exists.
+bool series_chosen(const hmc_ctx* c);
+int series_ctx_init(hmc_ctx* c);
+int series_apply(const ChainView& v, const double* phi, const float2* in, float2* out, bool dag,
+                 cudaStream_t s);
+int series_cg(hmc_ctx* c, const double* phi, const double2* chi, double2* x, double tol,
+              int max_iter, cudaStream_t s);
+int series_trajectory(hmc_ctx* c, const TrajArgs& a, cudaStream_t s);
+// The series' batch kernel (512 threads, as many bytes of shared memory as *smem
+// receives); null on a CUDA error.
+const void* series_batch_kernel(unsigned* smem);
+constexpr int kSeriesThreads = 512;
+
 struct TcBatch;
 int tc_batch_create(const hmc_params* p, int n, TcBatch** out);
 void tc_batch_destroy(TcBatch* b);

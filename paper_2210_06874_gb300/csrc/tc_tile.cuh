@@ -306,6 +306,7 @@ struct TcState {
                        // barrier phases are counted on their own)
     uint32_t wtile;    // slice-major tiles so far
     uint32_t gseq;     // split-K: team words posted so far (sk_post)
+    const void* ser;   // series iterations: their ser::Work
     int sk_loaded;     // split-K: this CTA's part of E' is resident
     uint32_t nskb;     // split-K CG: applications whose sources came by TMA (skb phases)
     int* status;

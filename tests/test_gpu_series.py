@@ -49,3 +49,54 @@ def test_fp64_against_oracle(L, Nt, kappa, delta, mu):
         x, st = c.cg_solve(dev(phi), dev(psi), tol=1e-12)
         r = psi - ops.apply_MMdag(E, phi, x.cpu().numpy())
         assert st.status == 0 and np.linalg.norm(r) < 1e-11 * np.linalg.norm(psi)
+
+
+# mixed path, automatic choice: (L, Nt, team_ctas, kappa, delta, mu) -- one CTA
+# with its vectors in registers and in memory, clusters, global-memory teams,
+# one and two cells per thread, several and ragged slices per CTA, one slice, and
+# the lattices and delta kappa beyond which the tensor-core tiles take over
+MIXED = [(1, 1, 0, 1.0, 0.125, 0.0), (1, 3, 1, 1.0, 0.125, 0.0), (2, 1, 0, 1.0, 0.125, 0.0),
+         (3, 8, 0, 1.0, 0.25, 0.0), (3, 8, 1, 1.0, 0.25, 0.3), (4, 5, 3, -1.0, 0.125, 0.0),
+         (3, 200, 0, 1.0, 0.05, 0.0), (6, 32, 0, 1.0, 0.125, 0.0), (6, 32, 3, 1.0, 0.125, 0.0),
+         (5, 7, 0, 0.0, 0.125, 0.0), (9, 20, 0, 1.0, 0.125, 0.0), (9, 37, 0, 1.0, 0.125, 0.0),
+         (12, 33, 1, 1.0, 0.125, 0.0), (16, 6, 2, 1.0, 0.125, 0.0), (17, 18, 0, 1.0, 0.125, 0.0),
+         (23, 4, 0, 1.0, 0.125, 0.0), (27, 3, 0, 1.0, 0.125, 0.0), (28, 2, 0, 1.0, 0.125, 0.0),
+         (4, 6, 0, 1.0, 1.4, 0.0)]
+
+
+@pytest.mark.parametrize("L,Nt,team,kappa,delta,mu", MIXED)
+def test_mixed_against_oracle(L, Nt, team, kappa, delta, mu):
+    """Applications to 2e-6 (the bound of every mixed application) and a solve to
+    the FP64 residual 1e-10, twice with the same bits."""
+    V, U = 2 * L * L, 2.0
+    c = hmc.Context(hmc.Params(L=L, Nt=Nt, kappa=kappa, beta=delta * Nt, U=U, mu=mu,
+                               team_ctas=team, precision=hmc.PREC_MIXED))
+    E = np.exp(-delta * mu) * ops.transfer_matrix(lattice.hopping_matrix(L), delta * kappa)
+    phi = synth.gaussian_field(910 + L, Nt, V, delta * U, scale=0.3)
+    psi = synth.complex_gaussian(911 + L, Nt, V)
+    p32 = dev(psi).to(torch.complex64)
+    seen = p32.cpu().numpy().astype(np.complex128)
+    tol = 2e-6 * max(1.0, np.exp(6 * abs(delta * kappa) - 1.5))
+    assert rel(c.apply_M(dev(phi), p32, prec=hmc.PREC_MIXED).cpu().numpy(),
+               ops.apply_M(E, phi, seen)) < tol
+    assert rel(c.apply_Mdag(dev(phi), p32, prec=hmc.PREC_MIXED).cpu().numpy(),
+               ops.apply_Mdag(E, phi, seen)) < tol
+    if delta > 1.0:
+        return
+    x, st = c.cg_solve(dev(phi), dev(psi), tol=1e-10, prec=hmc.PREC_MIXED)
+    r = psi - ops.apply_MMdag(E, phi, x.cpu().numpy())
+    assert st.status == 0 and np.linalg.norm(r) < 1.2e-10 * np.linalg.norm(psi)
+    x2, st2 = c.cg_solve(dev(phi), dev(psi), tol=1e-10, prec=hmc.PREC_MIXED)
+    assert st2.iterations == st.iterations and torch.equal(x, x2)
+
+
+def test_mixed_trajectory_follows_the_fp64_one():
+    """A trajectory on the automatic choice against the plain FP64 path's."""
+    L, Nt = 9, 21
+    kw = dict(L=L, Nt=Nt, beta=0.125 * Nt, U=3.0, n_md=4, traj_length=0.4)
+    phi = dev(synth.gaussian_field(77, Nt, 2 * L * L, 0.375, scale=0.4))
+    a, b = phi.clone(), phi.clone()
+    oa = hmc.Context(hmc.Params(cg_tol=1e-10, precision=hmc.PREC_MIXED, **kw)).trajectory(a, 3, 1)
+    ob = hmc.Context(hmc.Params(cg_tol=1e-12, **kw)).trajectory(b, 3, 1)
+    assert oa.status == 0 and oa.accept == ob.accept and abs(oa.dH - ob.dH) < 1e-7
+    assert rel(a.cpu().numpy(), b.cpu().numpy()) < 1e-8
