@@ -147,12 +147,12 @@ __device__ __forceinline__ double finish(const ChainView& c, int t, size_t o, do
 // A thread's cells of the tile (cell j = tid + j blockDim of the tile's
 // slices, both sublattices): the A site's index in the hop buffer and those of
 // the neighbours that are not in the cell.
-constexpr int kCells = 4;
+template <int NC>
 struct Cells {
     int n;                                    // cells of the tile
-    int a[kCells];                            // A site (its B site: a + LL)
-    int bm1[kCells], bm2[kCells];             // B(m1-1, m2), B(m1, m2-1)
-    int ap1[kCells], ap2[kCells];             // A(m1+1, m2), A(m1, m2+1)
+    int a[NC];                                // A site (its B site: a + LL)
+    int bm1[NC], bm2[NC];                     // B(m1-1, m2), B(m1, m2-1)
+    int ap1[NC], ap2[NC];                     // A(m1+1, m2), A(m1, m2+1)
     __device__ __forceinline__ bool has(int j) const {
         return (int)(threadIdx.x + j * blockDim.x) < n;
     }
@@ -160,7 +160,7 @@ struct Cells {
         const int LL = L * L, V = 2 * LL;
         n = ns * LL;
 #pragma unroll
-        for (int j = 0; j < kCells; ++j) {
+        for (int j = 0; j < NC; ++j) {
             const int cell = threadIdx.x + j * blockDim.x;
             if (!has(j)) continue;
             const int s = cell / LL, cc = cell - s * LL, m1 = cc / L, m2 = cc - m1 * L;
@@ -180,13 +180,13 @@ struct Cells {
 // and more for a warp's six FP64 instructions per cell).  E is real, so the two
 // components are independent; one at a time halves the registers and the
 // buffer.
-__device__ __forceinline__ void hop_horner(const HopSeries& hs, const Cells& cl, int LL,
-                                           double* y, double (&vA)[kCells],
-                                           double (&vB)[kCells]) {
-    double yA[kCells], yB[kCells];
+template <int NC>
+__device__ __forceinline__ void hop_horner(const HopSeries& hs, const Cells<NC>& cl, int LL,
+                                           double* y, double (&vA)[NC], double (&vB)[NC]) {
+    double yA[NC], yB[NC];
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < kCells; ++j)
+    for (int j = 0; j < NC; ++j)
         if (cl.has(j)) {
             yA[j] = vA[j];
             yB[j] = vB[j];
@@ -197,7 +197,7 @@ __device__ __forceinline__ void hop_horner(const HopSeries& hs, const Cells& cl,
         const double r = hs.r64[k - 1];
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < kCells; ++j)
+        for (int j = 0; j < NC; ++j)
             if (cl.has(j)) {
                 const double sA = (yB[j] + y[cl.bm1[j]]) + y[cl.bm2[j]];
                 const double sB = (yA[j] + y[cl.ap1[j]]) + y[cl.ap2[j]];
@@ -207,14 +207,14 @@ __device__ __forceinline__ void hop_horner(const HopSeries& hs, const Cells& cl,
         if (k == 1) break;
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < kCells; ++j)
+        for (int j = 0; j < NC; ++j)
             if (cl.has(j)) {
                 y[cl.a[j]] = yA[j];
                 y[cl.a[j] + LL] = yB[j];
             }
     }
 #pragma unroll
-    for (int j = 0; j < kCells; ++j) {
+    for (int j = 0; j < NC; ++j) {
         vA[j] = yA[j];
         vB[j] = yB[j];
     }
@@ -226,20 +226,20 @@ __host__ __device__ inline bool series_form(const ChainView& c, int doubles) {
 
 // Slices per series tile on a hop buffer of `doubles`: enough to give every
 // CTA of the team a tile, at most what the buffer and the threads take.
-__device__ __forceinline__ int series_slices(const ChainView& c, int team, int doubles) {
+__device__ __forceinline__ int series_slices(const ChainView& c, int team, int doubles, int cells) {
     const int LL = c.V / 2;
-    const int most = min(kCells * (int)blockDim.x / LL, doubles / c.V);
+    const int most = min(cells * (int)blockDim.x / LL, doubles / c.V);
     return max(1, min(most, (c.Nt + team - 1) / team));
 }
 
 // One tile of ns slices from t0 on by the series.  PHASES: e^{i phi} is
 // computed here from ea.phi (standalone applications) instead of read from
 // c.cis.  buf: ns V doubles.
-template <bool DAG, int EPI, bool PHASES = false>
+template <bool DAG, int EPI, int NC, bool PHASES = false>
 __device__ double series_tile(const ChainView& c, int t0, int ns, const double2* in, double2* out,
                               const EpiArgs& ea, double* buf) {
     const int V = c.V, LL = V / 2, Nt = c.Nt;
-    Cells cl;
+    Cells<NC> cl;
     cl.init(c.L, ns);
     auto phase = [&](size_t o) {
         if (!PHASES) return c.cis[o];
@@ -247,9 +247,9 @@ __device__ double series_tile(const ChainView& c, int t0, int ns, const double2*
         sincos(ea.phi[o], &sn, &cs);
         return make_double2(cs, sn);
     };
-    double2 vA[kCells], vB[kCells];
+    double2 vA[NC], vB[NC];
 #pragma unroll
-    for (int j = 0; j < kCells; ++j)
+    for (int j = 0; j < NC; ++j)
         if (cl.has(j)) {
             const int s = ns == 1 ? 0 : cl.a[j] / V, t = t0 + s;
             const int ts = DAG ? (t + 1 == Nt ? 0 : t + 1) : (t == 0 ? Nt - 1 : t - 1);
@@ -261,22 +261,22 @@ __device__ double series_tile(const ChainView& c, int t0, int ns, const double2*
                 vB[j] = cmul(phase(o + LL), vB[j]);
             }
         }
-    double a[kCells], b[kCells];
+    double a[NC], b[NC];
 #pragma unroll
-    for (int j = 0; j < kCells; ++j) { a[j] = vA[j].x; b[j] = vB[j].x; }
+    for (int j = 0; j < NC; ++j) { a[j] = vA[j].x; b[j] = vB[j].x; }
     hop_horner(c.ser, cl, LL, buf, a, b);
 #pragma unroll
-    for (int j = 0; j < kCells; ++j) {
+    for (int j = 0; j < NC; ++j) {
         vA[j].x = a[j]; vB[j].x = b[j];
         a[j] = vA[j].y; b[j] = vB[j].y;
     }
     hop_horner(c.ser, cl, LL, buf, a, b);
 #pragma unroll
-    for (int j = 0; j < kCells; ++j) { vA[j].y = a[j]; vB[j].y = b[j]; }
+    for (int j = 0; j < NC; ++j) { vA[j].y = a[j]; vB[j].y = b[j]; }
     const double hop = (1.0 + ea.hop_m1) * c.ser.c0;
     double acc = 0.0;
 #pragma unroll
-    for (int j = 0; j < kCells; ++j)
+    for (int j = 0; j < NC; ++j)
         if (cl.has(j)) {
             const int s = ns == 1 ? 0 : cl.a[j] / V, t = t0 + s;
             const size_t o = (size_t)t0 * V + cl.a[j];
@@ -356,8 +356,10 @@ __device__ double apply_tile(const ChainView& c, int tile, const double2* __rest
                             DAG ? cis[o] : make_double2(1.0, 0.0), in, out, ea);
 }
 
-// Which form of E a kernel is compiled with: FORM_EITHER decides per chain.
-enum Form : int { FORM_DENSE = 0, FORM_SERIES = 1, FORM_EITHER = 2 };
+// Which form of E a kernel is compiled with: FORM_EITHER decides per chain;
+// FORM_WIDE is the series in blocks of up to 640 threads with at least half a
+// thread per cell of a slice (series_cg.cuh).
+enum Form : int { FORM_DENSE = 0, FORM_SERIES = 1, FORM_EITHER = 2, FORM_WIDE = 3 };
 
 template <bool DAG, int EPI>
 __device__ __forceinline__ double dense_team(const ChainView& c, const Team& tm,
@@ -380,9 +382,12 @@ __device__ __noinline__ double series_team(const ChainView& c, const Team tm, co
     if (FORM == FORM_EITHER && !series_form(c, kHopDoubles))
         return dense_team<DAG, EPI>(c, tm, in, out, ea, sm);
     double acc = 0.0;
-    const int ns = series_slices(c, tm.size, kHopDoubles);
+    // (V <= kHopDoubles: at most 768 cells; 256 threads, or at least half of
+    // the cells)
+    constexpr int NC = FORM == FORM_WIDE ? 2 : 3;
+    const int ns = series_slices(c, tm.size, kHopDoubles, NC);
     for (int t0 = tm.rank * ns; t0 < c.Nt; t0 += tm.size * ns)
-        acc += series_tile<DAG, EPI>(c, t0, min(ns, c.Nt - t0), in, out, ea, &sm.Et[0][0]);
+        acc += series_tile<DAG, EPI, NC>(c, t0, min(ns, c.Nt - t0), in, out, ea, &sm.Et[0][0]);
     return acc;
 }
 

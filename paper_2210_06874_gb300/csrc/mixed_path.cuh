@@ -302,7 +302,7 @@ struct PersistentArgs {
 enum TileKind : int { kKindSite = 0, kKindSmall = 1, kKindSlice = 2, kKindSplitK = 3,
                       kKindSeries = 4 };
 template <int KIND>
-constexpr int kForm = KIND == kKindSeries   ? f64::FORM_SERIES
+constexpr int kForm = KIND == kKindSeries   ? f64::FORM_WIDE
                       : KIND == kKindSplitK ? f64::FORM_EITHER
                                             : f64::FORM_DENSE;
 

@@ -14,42 +14,42 @@
 namespace hmc {
 namespace ser {
 
+constexpr int kApplyThreads = 576;   // L = 24: one cell per thread
+
 // Standalone application, target slice blockIdx.x: the source slice's phase is
 // computed here, the slice hopped in shared memory (two buffers of V float2)
 // and the result formed: the vector, phi and the output each move once.
 template <bool DAG, int N>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kApplyThreads)
     k_apply(const __grid_constant__ ChainView c, const double* __restrict__ phi,
             const float2* __restrict__ in, float2* __restrict__ out) {
-    extern __shared__ __align__(16) uint8_t dyn[];
     const int V = c.V, LL = V / 2, Nt = c.Nt, t = blockIdx.x;
     const int ts = DAG ? (t + 1 == Nt ? 0 : t + 1) : (t == 0 ? Nt - 1 : t - 1);
     const float2* src = in + (size_t)ts * V;
     const size_t o = (size_t)t * V;
     const double* ph = phi + (DAG ? o : (size_t)ts * V);
     Cells<N> cl;
-    cl.init(c.L, 1);
+    cl.init(c.L, 1, blockDim.x);
     float4 v[N], cis[N], self[N];
 #pragma unroll
     for (int j = 0; j < N; ++j)
         if (cl.has(j)) {
-            const int a = cl.a[j];
-            const float2 u = src[a], w = src[a + LL], p = in[o + a], q = in[o + a + LL];
+            const int a = cl.cell(j);
+            v[j] = field_cell(src, a, LL);
+            self[j] = field_cell(in + o, a, LL);
             float sa, ca, sb, cb;
             sincosf((float)ph[a], &sa, &ca);
             sincosf((float)ph[a + LL], &sb, &cb);
             cis[j] = make_float4(ca, sa, cb, sb);
-            v[j] = make_float4(u.x, u.y, w.x, w.y);
-            self[j] = make_float4(p.x, p.y, q.x, q.y);
             if (!DAG) v[j] = phase4<false>(cis[j], v[j]);
         }
     int par = 0;
-    hop<N>(c.ser.r32, c.ser.k32, cl, LL, reinterpret_cast<float2*>(dyn), V, par, v);
+    hop<N>(c.ser.r32, c.ser.k32, cl, reinterpret_cast<float4*>(ser_dyn), LL, par, v, [] {});
     const float c0 = c.ser.c0f, sg = (DAG ? t == Nt - 1 : t == 0) ? c0 : -c0;
 #pragma unroll
     for (int j = 0; j < N; ++j)
         if (cl.has(j)) {
-            const int a = cl.a[j];
+            const int a = cl.cell(j);
             const float4 w = axpy4(sg, DAG ? phase4<true>(cis[j], v[j]) : v[j], self[j]);
             out[o + a] = make_float2(w.x, w.y);
             out[o + a + LL] = make_float2(w.z, w.w);
@@ -63,19 +63,16 @@ struct Launch {
     int cluster;        // the grid is one cluster of this many CTAs (0: global team)
     unsigned smem;      // dynamic shared memory in bytes
 };
-__device__ __forceinline__ Team begin(const ChainView& c, const Launch& la, uint8_t* dyn,
-                                      ClusterSync* cs, uint64_t* norm, float* ratio,
-                                      unsigned* seq, Work& wk) {
+__device__ __forceinline__ Team begin(const ChainView& c, const Launch& la, ClusterSync* cs,
+                                      uint64_t* norm, unsigned* seq, Work& wk) {
     Team tm = tc::make_team(c);
-    wk.smem = dyn;
     wk.bytes = la.smem;
     wk.mail_V = la.cluster ? c.V : 0;
     wk.norm_smem = norm;
-    wk.ratio = ratio;
     wk.seq = seq;
     if (threadIdx.x == 0) *seq = *c.ser_seq;
     if (la.cluster) {
-        uint64_t* m = reinterpret_cast<uint64_t*>(dyn);
+        uint64_t* m = reinterpret_cast<uint64_t*>(ser_dyn);
         for (int i = threadIdx.x; i < (int)(mail_bytes(c.V) / 8); i += blockDim.x) m[i] = 0;
         if (threadIdx.x < 32) norm[threadIdx.x] = 0;
         __syncthreads();
@@ -94,14 +91,12 @@ __device__ __forceinline__ void end(const ChainView& c, const Launch& la, const 
 }
 
 #define HMC_SER_BEGIN()                                                                   \
-    extern __shared__ __align__(16) uint8_t dyn[];                                        \
     __shared__ f64::Smem sm64;                                                            \
     __shared__ ClusterSync s_cs;                                                          \
     __shared__ uint64_t s_norm[32];                                                       \
-    __shared__ float s_ratio[kSerMax32];                                                  \
     __shared__ unsigned s_seq;                                                            \
     Work wk;                                                                              \
-    Team tm = begin(c, la, dyn, &s_cs, s_norm, s_ratio, &s_seq, wk);                      \
+    Team tm = begin(c, la, &s_cs, s_norm, &s_seq, wk);                                    \
     tc::TcState st;                                                                       \
     st.ser = &wk
 
@@ -144,15 +139,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     k_batch(const tc::BatchItem* __restrict__ items, const int* __restrict__ order, int n,
             int* queue, const tc::BatchCallArgs* call, double* outs, int csize, int mail_V,
             unsigned smem) {
-    extern __shared__ __align__(16) uint8_t dyn[];
     __shared__ f64::Smem sm64;
     __shared__ ClusterSync s_cs;
     __shared__ uint64_t s_norm[32];
-    __shared__ float s_ratio[kSerMax32];
     __shared__ unsigned s_seq;
-    Work wk{dyn, smem, mail_V, s_norm, s_ratio, &s_seq};
+    Work wk{smem, mail_V, s_norm, &s_seq};
     if (threadIdx.x == 0) s_seq = 0;
-    uint64_t* m = reinterpret_cast<uint64_t*>(dyn);
+    uint64_t* m = reinterpret_cast<uint64_t*>(ser_dyn);
     for (int i = threadIdx.x; i < (int)(mail_bytes(mail_V) / 8); i += blockDim.x) m[i] = 0;
     if (threadIdx.x < 32) s_norm[threadIdx.x] = 0;
     __syncthreads();
@@ -234,8 +227,8 @@ int series_ctx_init(hmc_ctx* c) {
 int series_apply(const ChainView& v, const double* phi, const float2* in, float2* out, bool dag,
                  cudaStream_t s) {
     const int LL = v.V / 2;
-    const bool two = LL > ser::kThreads;
-    const int thr = ser::threads(v.L, 1, 1);
+    const bool two = LL > ser::kApplyThreads;
+    const int thr = ((two ? (LL + 1) / 2 : LL) + 31) / 32 * 32;
     const size_t smem = 2 * (size_t)v.V * sizeof(float2);
     if (dag && two) ser::k_apply<true, 2><<<v.Nt, thr, smem, s>>>(v, phi, in, out);
     else if (dag) ser::k_apply<true, 1><<<v.Nt, thr, smem, s>>>(v, phi, in, out);
@@ -263,18 +256,15 @@ static int launch_series(hmc_ctx* c, const void* fn, tc::PersistentArgs& pa, ser
         la.cluster = cluster ? T : 0;
         pa.inner = T;
         pa.cluster = 0;
-        const int thr = ser::threads(v.L, v.Nt, T);
-        const ser::Shape sh = ser::shape(v.L, v.Nt, T, thr);
-        const size_t vec = (size_t)sh.S * v.V * sizeof(float2);
+        const ser::Shape sh = ser::shape(v.L, v.Nt, T);
         cudaFuncAttributes at;
         if (cudaFuncGetAttributes(&at, fn) != cudaSuccess) return HMC_ERR_CUDA;
-        const size_t want = ser::mail_bytes(cluster ? v.V : 0) + ser::hop_bytes(v.V, sh) +
-                            vec * (sh.reg ? 1 : 7);
+        const size_t want = ser::shared_bytes(v.V, cluster ? v.V : 0, sh, ser::kVecs + 1);
         la.smem = (unsigned)std::min(want, (size_t)at.maxDynamicSharedSizeBytes);
         if (!control_reset(v, T, s)) return HMC_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(T);
-        cfg.blockDim = dim3(thr);
+        cfg.blockDim = dim3(sh.workers + 32);   // the service warp
         cfg.dynamicSmemBytes = la.smem;
         cfg.stream = s;
         cudaLaunchAttribute a[1];
