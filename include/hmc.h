@@ -85,7 +85,10 @@ typedef struct hmc_params {
     int team_ctas;       /* CTAs of a persistent launch (0: automatic); in a
                             batch, 2..8 runs the chain on a thread-block
                             cluster of that many CTAs (one size per batch;
-                            those chains go first), else one CTA */
+                            those chains go first), 1 on one CTA, 0 on one
+                            CTA or, where that shortens the step and every
+                            chain is on the automatic operand mode, on a
+                            cluster of 8 (chains of over 2048 sites) */
     int tile_slices;     /* time slices per tensor-core tile, one of 8, 16, 32
                             (operand_mode 4: 1..64; 0: automatic) */
     int inner_ctas;      /* CTAs running the FP32 iterations of the mixed CG

@@ -9,6 +9,8 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
+#include <queue>
 #include <vector>
 
 #include "mixed_path.cuh"
@@ -1308,6 +1310,97 @@ void tc_batch_destroy(TcBatch* b) {
     delete b;
 }
 
+// Makespan of a batch step as the kernel schedules it: the first k of the chains
+// `order` (by decreasing cost) as cluster teams, each taken by the next free
+// cluster of csize CTAs, whose CTAs then take one-CTA chains on their own.
+static double series_makespan(const std::vector<double>& solo, const std::vector<double>& team,
+                              const std::vector<int>& order, const std::vector<char>& is_team,
+                              int clusters, int csize) {
+    using Heap = std::priority_queue<double, std::vector<double>, std::greater<double>>;
+    Heap clu(std::greater<double>(), std::vector<double>(clusters, 0.0));
+    double end = 0.0;
+    for (int i : order)
+        if (is_team[i]) {
+            const double t = clu.top() + team[i];
+            clu.pop();
+            clu.push(t);
+            end = std::max(end, t);
+        }
+    std::vector<double> start;
+    for (; !clu.empty(); clu.pop()) start.insert(start.end(), csize, clu.top());
+    Heap cta(std::greater<double>(), std::move(start));
+    for (int i : order)
+        if (!is_team[i]) {
+            const double t = cta.top() + solo[i];
+            cta.pop();
+            cta.push(t);
+            end = std::max(end, t);
+        }
+    return end;
+}
+
+// Cluster teams of a series batch that asks for none (team_ctas 0 or 1 is one CTA
+// when given; 0 leaves it to the library): chains whose vectors do not fit one
+// CTA's shared memory may run on 8 CTAs, as many of the largest as shorten the
+// step.  Clocks per half iteration, measured (L = 6, Nt = 32 and L = 12, Nt = 64
+// on one CTA: 12,900 and 104,000; the latter on 8 CTAs: 14,200): 5.6 a site, plus
+// 2,500 for a team's exchange; iterations grow in proportion to Nt delta.
+static void plan_series_teams(TcBatch* b, std::vector<char>& is_team) {
+    constexpr int kTeam = 8, kSoloSites = 2048;
+    const int n = b->n;
+    std::vector<double> solo(n), team(n);
+    std::vector<int> order(n), cand;
+    for (int i = 0; i < n; ++i) {
+        const hmc_params& p = b->ctxs[i]->params;
+        if (p.team_ctas > 1) return;                 // the caller chose
+        const double its = p.beta * p.n_md * (p.integrator == 1 ? 2 : 1);
+        const double sites = b->ctxs[i]->view.N;
+        solo[i] = its * (500.0 + 5.6 * sites);
+        team[i] = its * (2500.0 + 5.6 * sites / kTeam);
+        order[i] = i;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return solo[x] > solo[y]; });
+    for (int i : order)
+        if (b->ctxs[i]->params.team_ctas == 0 && b->ctxs[i]->view.N > kSoloSites &&
+            b->ctxs[i]->params.Nt >= kTeam)
+            cand.push_back(i);
+    if (cand.empty()) return;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(b->ctxs[0]->num_sms / kTeam * kTeam);
+    cfg.blockDim = dim3(b->threads);
+    cfg.dynamicSmemBytes = b->smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kTeam;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, b->kernel, &cfg) != cudaSuccess ||
+        clusters < 1) {
+        (void)cudaGetLastError();
+        return;
+    }
+    // without teams every SM takes one-CTA chains
+    std::vector<char> none(n, 0);
+    double best = series_makespan(solo, team, order, none, b->ctxs[0]->num_sms, 1);
+    size_t best_k = 0;
+    const size_t step = std::max<size_t>(1, cand.size() / 48);
+    std::vector<char> flags(n, 0);
+    for (size_t k = 0; k < cand.size();) {
+        for (size_t q = 0; q < step && k < cand.size(); ++q) flags[cand[k++]] = 1;
+        const double m = series_makespan(solo, team, order, flags, clusters, kTeam);
+        if (m < best) {
+            best = m;
+            best_k = k;
+        }
+    }
+    for (size_t k = 0; k < best_k; ++k) {
+        is_team[cand[k]] = 1;
+        b->ctxs[cand[k]]->params.team_ctas = kTeam;
+    }
+}
+
 int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
     TcBatch* b = new TcBatch();
     b->n = n;
@@ -1352,6 +1445,8 @@ int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
             return HMC_ERR_CUDA;
         }
     }
+    std::vector<char> auto_team(n, 0);
+    if (b->series) plan_series_teams(b, auto_team);
     std::vector<CUtensorMap> maps(4 * n_maps);
     for (int i = 0; i < n; ++i)
         if (leader[i] == i) {
@@ -1363,7 +1458,7 @@ int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
     // chains asking for a team (team_ctas >= 2) run on a thread-block
     // cluster of that many CTAs; all such chains of a batch use one size
     for (int i = 0; i < n; ++i) {
-        const int tmc = p[i].team_ctas;
+        const int tmc = b->ctxs[i]->params.team_ctas;
         if (tmc <= 1) continue;
         if (tmc > tc::kMaxClusterW || (b->csize > 1 && tmc != b->csize)) {
             tc_batch_destroy(b);
@@ -1388,7 +1483,10 @@ int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
         it.team = c->params.team_ctas > 1 ? c->params.team_ctas : 1;
         it.pa.inner = 1;
         it.pa.cluster = 0;
-        if (it.team > 1) {
+        if (it.team > 1 && auto_team[i]) {
+            it.pa = tc::PersistentArgs{};
+            it.pa.inner = it.pa.cluster = it.team;
+        } else if (it.team > 1) {
             // a cluster team: the launch shape of a single-chain run on
             // team CTAs with an inner team of all of them, as one cluster
             if (c->params.inner_ctas == 0) c->params.inner_ctas = it.team;

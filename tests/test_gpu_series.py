@@ -100,3 +100,23 @@ def test_mixed_trajectory_follows_the_fp64_one():
     ob = hmc.Context(hmc.Params(cg_tol=1e-12, **kw)).trajectory(b, 3, 1)
     assert oa.status == 0 and oa.accept == ob.accept and abs(oa.dH - ob.dH) < 1e-7
     assert rel(a.cpu().numpy(), b.cpu().numpy()) < 1e-8
+
+
+def test_batch_puts_large_chains_on_clusters():
+    """A batch that leaves the teams to the library runs its chains of over 2048
+    sites on clusters of 8 CTAs: against the FP64 path from the same fields."""
+    sizes = [(12, 24, 3.0), (3, 8, 2.0), (9, 16, 4.0), (9, 15, 3.5), (24, 4, 3.0)]
+    kw = [dict(L=L, Nt=Nt, U=U, beta=0.125 * Nt, n_md=3, traj_length=0.3) for L, Nt, U in sizes]
+    b = hmc.Batch([hmc.Params(cg_tol=1e-10, precision=hmc.PREC_MIXED, **k) for k in kw])
+    phi = torch.zeros(b.total, dtype=torch.float64, device=DEV)
+    starts = [dev(synth.gaussian_field(80 + i, Nt, 2 * L * L, 0.125 * U, scale=0.4))
+              for i, (L, Nt, U) in enumerate(sizes)]
+    for i, f in enumerate(starts):
+        b.view(phi, i).copy_(f)
+    outs = b.trajectory(phi, 21, 2)
+    for i, k in enumerate(kw):
+        want = starts[i].clone()
+        o = hmc.Context(hmc.Params(cg_tol=1e-12, **k)).trajectory(want, 21, 2, chain=i)
+        assert outs[i].status == 0 and outs[i].max_true_residual <= 1e-10
+        assert outs[i].accept == o.accept and abs(outs[i].dH - o.dH) < 1e-7
+        assert rel(b.view(phi, i).cpu().numpy(), want.cpu().numpy()) < 1e-8
