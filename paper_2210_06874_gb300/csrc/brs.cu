@@ -22,25 +22,10 @@
 namespace hmc {
 namespace brs {
 
-template <typename T>
-struct C2;
-template <>
-struct C2<double> {
-    using type = double2;
-};
-template <>
-struct C2<float> {
-    using type = float2;
-};
-
-template <typename T>
-__device__ __forceinline__ typename C2<T>::type cm(typename C2<T>::type a,
-                                                   typename C2<T>::type b) {
+__device__ __forceinline__ float2 cm(float2 a, float2 b) {
     return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
 }
-template <typename T>
-__device__ __forceinline__ typename C2<T>::type cmc(typename C2<T>::type a,
-                                                    typename C2<T>::type b) {  // conj(a) b
+__device__ __forceinline__ float2 cmc(float2 a, float2 b) {  // conj(a) b
     return {a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x};
 }
 
@@ -56,12 +41,11 @@ __global__ void k_phases(const double* __restrict__ phi, double2* __restrict__ c
     }
 }
 
-// One output site-slice; blockIdx.y is the slice, so no 64-bit division.
-template <typename T, bool DAG>
-__device__ __forceinline__ typename C2<T>::type site(int L, int LL, int V, int Nt, int t, int x,
-                                                     T dk, const typename C2<T>::type* cis,
-                                                     const typename C2<T>::type* in) {
-    using T2 = typename C2<T>::type;
+// One output site-slice (FP32, any L); blockIdx.y is the slice, so no 64-bit division.
+template <bool DAG>
+__device__ __forceinline__ float2 site(int L, int LL, int V, int Nt, int t, int x, float dk,
+                                       const float2* cis, const float2* in) {
+    using T2 = float2;
     const bool isB = x >= LL;
     const int cidx = isB ? x - LL : x;
     const int m1 = cidx / L, m2 = cidx - m1 * L;
@@ -80,13 +64,13 @@ __device__ __forceinline__ typename C2<T>::type site(int L, int LL, int V, int N
     const T2 self = row[x];
     const bool up = DAG ? isB : !isB;   // forward time neighbour needed
     int tn;
-    T sg = (T)1;
+    float sg = 1.f;
     if (up) {
         tn = t + 1;
-        if (tn == Nt) { tn = 0; sg = (T)-1; }
+        if (tn == Nt) { tn = 0; sg = -1.f; }
     } else {
         tn = t - 1;
-        if (tn < 0) { tn = Nt - 1; sg = (T)-1; }
+        if (tn < 0) { tn = Nt - 1; sg = -1.f; }
     }
     T2 nb = in[(size_t)tn * V + x];
     nb.x *= sg;
@@ -94,18 +78,18 @@ __device__ __forceinline__ typename C2<T>::type site(int L, int LL, int V, int N
     T2 r;
     if (!DAG) {
         if (!isB) {   // psi_{t+1} - e^{i phi_t} psi_t
-            const T2 w = cm<T>(cis[(size_t)t * V + x], self);
+            const T2 w = cm(cis[(size_t)t * V + x], self);
             r = {nb.x - w.x, nb.y - w.y};
         } else {      // psi_t - e^{-i phi_t} psi_{t-1}
-            const T2 w = cmc<T>(cis[(size_t)t * V + x], nb);
+            const T2 w = cmc(cis[(size_t)t * V + x], nb);
             r = {self.x - w.x, self.y - w.y};
         }
     } else {
         if (!isB) {   // psi_{t-1} - e^{-i phi_t} psi_t
-            const T2 w = cmc<T>(cis[(size_t)t * V + x], self);
+            const T2 w = cmc(cis[(size_t)t * V + x], self);
             r = {nb.x - w.x, nb.y - w.y};
         } else {      // psi_t - e^{i phi_{t+1}} psi_{t+1}  (phase of the wrapped t+1)
-            const T2 w = cm<T>(cis[(size_t)tn * V + x], nb);
+            const T2 w = cm(cis[(size_t)tn * V + x], nb);
             r = {self.x - w.x, self.y - w.y};
         }
     }
@@ -113,18 +97,18 @@ __device__ __forceinline__ typename C2<T>::type site(int L, int LL, int V, int N
 }
 
 // grid (ceil(V / (2*256)), Nt): each thread writes two consecutive sites.
-template <typename T, bool DAG>
-__global__ void __launch_bounds__(256) k_apply(int L, int Nt, T dk,
-                                               const typename C2<T>::type* __restrict__ cis,
-                                               const typename C2<T>::type* __restrict__ in,
-                                               typename C2<T>::type* __restrict__ out) {
+template <bool DAG>
+__global__ void __launch_bounds__(256) k_apply(int L, int Nt, float dk,
+                                               const float2* __restrict__ cis,
+                                               const float2* __restrict__ in,
+                                               float2* __restrict__ out) {
     const int LL = L * L, V = 2 * LL;
     const int t = blockIdx.y;
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x0 >= V) return;
-    typename C2<T>::type* o = out + (size_t)t * V;
-    o[x0] = site<T, DAG>(L, LL, V, Nt, t, x0, dk, cis, in);
-    if (x0 + 1 < V) o[x0 + 1] = site<T, DAG>(L, LL, V, Nt, t, x0 + 1, dk, cis, in);
+    float2* o = out + (size_t)t * V;
+    o[x0] = site<DAG>(L, LL, V, Nt, t, x0, dk, cis, in);
+    if (x0 + 1 < V) o[x0 + 1] = site<DAG>(L, LL, V, Nt, t, x0 + 1, dk, cis, in);
 }
 
 // FP32, even L: the two sites x0, x0+1 (x0 even) share a row of the
@@ -180,21 +164,21 @@ __global__ void __launch_bounds__(256) k_apply_f32_pairs(int L, int Nt, float dk
     const float2 c0 = make_float2(ph.x, ph.y), c1 = make_float2(ph.z, ph.w);
     if (!DAG) {
         if (!isB) {
-            const float2 u0 = cm<float>(c0, s0), u1 = cm<float>(c1, s1);
+            const float2 u0 = cm(c0, s0), u1 = cm(c1, s1);
             r0 = make_float2(b0.x - u0.x, b0.y - u0.y);
             r1 = make_float2(b1.x - u1.x, b1.y - u1.y);
         } else {
-            const float2 u0 = cmc<float>(c0, b0), u1 = cmc<float>(c1, b1);
+            const float2 u0 = cmc(c0, b0), u1 = cmc(c1, b1);
             r0 = make_float2(s0.x - u0.x, s0.y - u0.y);
             r1 = make_float2(s1.x - u1.x, s1.y - u1.y);
         }
     } else {
         if (!isB) {
-            const float2 u0 = cmc<float>(c0, s0), u1 = cmc<float>(c1, s1);
+            const float2 u0 = cmc(c0, s0), u1 = cmc(c1, s1);
             r0 = make_float2(b0.x - u0.x, b0.y - u0.y);
             r1 = make_float2(b1.x - u1.x, b1.y - u1.y);
         } else {
-            const float2 u0 = cm<float>(c0, b0), u1 = cm<float>(c1, b1);
+            const float2 u0 = cm(c0, b0), u1 = cm(c1, b1);
             r0 = make_float2(s0.x - u0.x, s0.y - u0.y);
             r1 = make_float2(s1.x - u1.x, s1.y - u1.y);
         }
@@ -203,6 +187,51 @@ __global__ void __launch_bounds__(256) k_apply_f32_pairs(int L, int Nt, float dk
     const float h1x = n0.z + n1.z + w1.x, h1y = n0.w + n1.w + w1.y;
     out[(size_t)t * V2 + p] =
         make_float4(r0.x - dk * h0x, r0.y - dk * h0y, r1.x - dk * h1x, r1.y - dk * h1y);
+}
+
+// FP64: bound by the FP64 issue rate (1.7 operations per clock and SM), so the
+// site is written in the ten operations it cannot do without -- four
+// multiply-adds for base - e^{+-i phi} w, four additions for the neighbours'
+// sum, two multiply-adds for -dk times it -- and signs are flipped in the
+// integer unit.  One site per thread: the branch on the sublattice is uniform in
+// all but one warp of a slice, and the loads of a warp are consecutive.  L = 51,
+// Nt = 100: 24.6 us with two sites per thread and 14 operations a site, 14.3 so.
+__device__ __forceinline__ double2 flip(double2 v, bool neg) {
+    const long long m = neg ? (long long)0x8000000000000000ull : 0ll;
+    return make_double2(__longlong_as_double(__double_as_longlong(v.x) ^ m),
+                        __longlong_as_double(__double_as_longlong(v.y) ^ m));
+}
+template <bool DAG>
+__global__ void __launch_bounds__(256) k_apply_f64(int L, int Nt, double mdk,
+                                                   const double2* __restrict__ cis,
+                                                   const double2* __restrict__ in,
+                                                   double2* __restrict__ out) {
+    const int LL = L * L, V = 2 * LL, t = blockIdx.y;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= V) return;
+    const bool isB = x >= LL;
+    const int c = isB ? x - LL : x;
+    const int m1 = c / L, m2 = c - m1 * L;
+    const double2* row = in + (size_t)t * V;
+    const double2* other = row + (isB ? 0 : LL);
+    // B(m1-1, m2), B(m1, m2-1) of an A site; A(m1+1, m2), A(m1, m2+1) of a B site
+    const int n1 = isB ? (m1 == L - 1 ? m2 : c + L) : (m1 == 0 ? c + LL - L : c - L);
+    const int n2 = isB ? (m2 == L - 1 ? c - (L - 1) : c + 1) : (m2 == 0 ? c + (L - 1) : c - 1);
+    const bool up = DAG == isB;   // forward time neighbour
+    const int tn = up ? (t + 1 == Nt ? 0 : t + 1) : (t == 0 ? Nt - 1 : t - 1);
+    const bool wrap = up ? t + 1 == Nt : t == 0;
+    const double2 self = row[x], nb = flip(in[(size_t)tn * V + x], wrap);
+    double2 ph = cis[(size_t)(DAG && isB ? tn : t) * V + x];
+    const double2 a = other[c], b1 = other[n1], b2 = other[n2];
+    // A: base = time neighbour, w = self; B: base = self, w = time neighbour.
+    // M: A e^{i phi}, B e^{-i phi}; M^dag: A e^{-i phi}, B e^{i phi}
+    const double2 base = isB ? self : nb, w = isB ? nb : self;
+    const double py = flip(make_double2(ph.y, 0.0), DAG != isB).x;
+    double rx = fma(-ph.x, w.x, base.x), ry = fma(-ph.x, w.y, base.y);
+    rx = fma(py, w.y, rx);
+    ry = fma(-py, w.x, ry);
+    const double hx = (a.x + b1.x) + b2.x, hy = (a.y + b1.y) + b2.y;
+    out[(size_t)t * V + x] = make_double2(fma(mdk, hx, rx), fma(mdk, hy, ry));
 }
 
 static int grid_for(long long N, int threads) {
@@ -238,12 +267,13 @@ int hmc_apply_brs(int L, int Nt, double delta_kappa, const void* cis, const void
     cudaStream_t s = (cudaStream_t)stream;
     using namespace hmc::brs;
     if (prec == HMC_PREC_FP64) {
+        const dim3 g1((V + 255) / 256, Nt);
         if (dagger)
-            k_apply<double, true><<<g, 256, 0, s>>>(L, Nt, delta_kappa, (const double2*)cis,
-                                                    (const double2*)in, (double2*)out);
+            k_apply_f64<true><<<g1, 256, 0, s>>>(L, Nt, -delta_kappa, (const double2*)cis,
+                                                 (const double2*)in, (double2*)out);
         else
-            k_apply<double, false><<<g, 256, 0, s>>>(L, Nt, delta_kappa, (const double2*)cis,
-                                                     (const double2*)in, (double2*)out);
+            k_apply_f64<false><<<g1, 256, 0, s>>>(L, Nt, -delta_kappa, (const double2*)cis,
+                                                  (const double2*)in, (double2*)out);
     } else if (prec == HMC_PREC_MIXED && (L % 2) == 0 &&
                ((reinterpret_cast<uintptr_t>(cis) | reinterpret_cast<uintptr_t>(in) |
                  reinterpret_cast<uintptr_t>(out)) & 15) == 0) {
@@ -258,10 +288,10 @@ int hmc_apply_brs(int L, int Nt, double delta_kappa, const void* cis, const void
                                                         (float4*)out);
     } else if (prec == HMC_PREC_MIXED) {
         if (dagger)
-            k_apply<float, true><<<g, 256, 0, s>>>(L, Nt, (float)delta_kappa, (const float2*)cis,
+            k_apply<true><<<g, 256, 0, s>>>(L, Nt, (float)delta_kappa, (const float2*)cis,
                                                    (const float2*)in, (float2*)out);
         else
-            k_apply<float, false><<<g, 256, 0, s>>>(L, Nt, (float)delta_kappa,
+            k_apply<false><<<g, 256, 0, s>>>(L, Nt, (float)delta_kappa,
                                                     (const float2*)cis, (const float2*)in,
                                                     (float2*)out);
     } else {
