@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(NTHR) k_apply_series(const __grid_constant__ C
     extern __shared__ __align__(16) double hop_buf[];
     EpiArgs ea = {};
     ea.phi = phi;
-    series_tile<DAG, EPI_STORE, true>(c, blockIdx.x, 1, in, out, ea, hop_buf);
+    series_tile<DAG, EPI_STORE, 4, true>(c, blockIdx.x, 1, in, out, ea, hop_buf);
 }
 
 __global__ void __launch_bounds__(NTHR) k_force_series(const __grid_constant__ ChainView c, const double* phi,
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(NTHR) k_force_series(const __grid_constant__ C
     ea.phi = phi;
     ea.F = F;
     ea.inv_dU = 1.0 / (c.delta * c.U);
-    series_tile<true, EPI_FORCE, true>(c, blockIdx.x, 1, x, nullptr, ea, hop_buf);
+    series_tile<true, EPI_FORCE, 4, true>(c, blockIdx.x, 1, x, nullptr, ea, hop_buf);
 }
 
 __device__ __forceinline__ Team make_team(const ChainView& c) {
