@@ -417,7 +417,7 @@ struct CgResult {
 // chi - M M^dag x then starts the iteration.  cis must hold exp(i phi).
 // The new direction p = r + beta p is formed inside the M^dag application, where
 // it is read and (into a second buffer) where it is owned, so an iteration has
-// two team sums and no barrier of its own for the direction.
+// two team sums and no barrier of its own for the direction (series).
 // Ends with the FP64 true residual, which leaves chi - M M^dag x in r and
 // M^dag x in q.
 template <int FORM>
@@ -431,7 +431,7 @@ __device__ inline bool cg_solve(const ChainView& c, Team& tm, const double2* chi
         if (!warm) {
             x[e] = make_double2(0.0, 0.0);
             r[e] = ch;
-            p[e] = make_double2(0.0, 0.0);
+            p[e] = FORM == FORM_DENSE ? ch : make_double2(0.0, 0.0);
         }
         v1[0] += ch.x * ch.x + ch.y * ch.y;
     }
@@ -459,21 +459,27 @@ __device__ inline bool cg_solve(const ChainView& c, Team& tm, const double2* chi
         double vr[1] = {apply_team<FORM, false, EPI_RESIDUAL>(c, tm, q, nullptr, ea, sm)};
         if (!team_sum<1>(tm, vr)) return false;
         rr = vr[0];
-        HMC_TEAM_ELEMS(e, c, tm) p[e] = make_double2(0.0, 0.0);
+        HMC_TEAM_ELEMS(e, c, tm) p[e] = FORM == FORM_DENSE ? r[e] : make_double2(0.0, 0.0);
         if (!team_barrier(tm)) return false;
         if (!finite_d(rr)) res.status = HMC_ERR_NONFINITE;
     }
     int it = 0;
     bool conv = res.status == HMC_OK && rr <= stop;
     while (!conv && res.status == HMC_OK && it < max_iter) {
-        // p = r + beta p, q = M^dag p
+        double vq[1];
         ea.p = p;
-        ea.p_new = pn;
-        double vq[1] = {apply_team<FORM, true, EPI_DIRECTION>(c, tm, r, q, ea, sm)};
-        if (!team_sum<1>(tm, vq)) return false;
-        pn = p;
-        p = ea.p_new;
-        ea.p = p;
+        if constexpr (FORM == FORM_DENSE) {
+            vq[0] = apply_team<FORM, true, EPI_STORE>(c, tm, p, q, ea, sm);   // q = M^dag p
+            if (!team_sum<1>(tm, vq)) return false;
+        } else {
+            // p = r + beta p, q = M^dag p
+            ea.p_new = pn;
+            vq[0] = apply_team<FORM, true, EPI_DIRECTION>(c, tm, r, q, ea, sm);
+            if (!team_sum<1>(tm, vq)) return false;
+            pn = p;
+            p = ea.p_new;
+            ea.p = p;
+        }
         const double qq = vq[0];
         if (!finite_d(qq) || !(qq > 0.0)) { res.status = HMC_ERR_NONFINITE; break; }
         ea.alpha = rr / qq;
@@ -485,6 +491,15 @@ __device__ inline bool cg_solve(const ChainView& c, Team& tm, const double2* chi
         if (rr_new <= stop) { conv = true; break; }
         ea.beta = rr_new / rr;
         rr = rr_new;
+        if constexpr (FORM == FORM_DENSE) {
+            // (the dense kernels run small lattices on one CTA: a barrier is cheap
+            // there, forming p twice in FP64 is not: 1.5 % of an L = 3 trajectory)
+            HMC_TEAM_ELEMS(e, c, tm) {
+                const double2 rv = r[e], pv = p[e];
+                p[e] = make_double2(fma(ea.beta, pv.x, rv.x), fma(ea.beta, pv.y, rv.y));
+            }
+            if (!team_barrier(tm)) return false;
+        }
     }
     res.iterations = it;
     if (res.status == HMC_OK && !conv) res.status = HMC_ERR_CG_NOT_CONVERGED;
