@@ -183,11 +183,23 @@ def workload_params(name, precision):
     return w, p, prec
 
 
-def flops_per_apply(V, Nt):
+def series_of(params, prec):
+    """Degree of the polynomial of the sparse hopping that an application runs
+    (0: the dense E)."""
+    from paper_2210_06874_gb300 import autotune
+    if not autotune.series_feasible(params):
+        return 0
+    rho = 3 * abs(params.delta * params.kappa)
+    if prec == "fp64":
+        return autotune.series_degree(rho, 2e-17) if params.V > 32 else 0
+    return autotune.series_degree(rho, 6e-9) if params.operand_mode == 0 else 0
+
+
+def flops_per_apply(V, Nt, degree=0):
     """Algorithmic FLOPs of one M or M^dag application: the real V x V by
-    V x 2Nt contraction (4 V^2 Nt) plus phase, shift and subtraction
-    (~10 V Nt)."""
-    return 4.0 * V * V * Nt + 10.0 * V * Nt
+    V x 2Nt contraction (4 V^2 Nt), or 8 per site and degree of the polynomial
+    of the sparse hopping, plus phase, shift and subtraction (~10 V Nt)."""
+    return (8.0 * degree if degree else 4.0 * V) * V * Nt + 10.0 * V * Nt
 
 
 
@@ -755,15 +767,16 @@ def run_ours(args):
     peaks, peaks_kind = load_peaks()
     mean_iters = statistics.mean(o.cg_iterations for o in outs)
     n_app = statistics.mean(applies_per_traj(o, params.n_md) for o in outs)
-    flop = n_app * flops_per_apply(V, Nt)
-    byts = n_app * apply_bytes(V, Nt, prec)
+    degree = series_of(params, prec)
+    flop = n_app * flops_per_apply(V, Nt, degree)
+    byts = n_app * apply_bytes(V, Nt, prec, degree)
     achieved = flop / (ms_per_step * 1e-3) / 1e12
     hbm_peak = peaks.get("hbm_gbs", FALLBACK["hbm_gbs"])
     traffic_it, traffic_src = committed_traffic(name, "per-cg-iteration")
     traffic = traffic_it * mean_iters if traffic_it is not None else None
     hbm = {"achieved_gbs": byts / (ms_per_step * 1e-3) / 1e9, "peak_gbs": hbm_peak,
            "algorithmic_bytes": byts,
-           "bytes_per_application": apply_bytes(V, Nt, prec),
+           "bytes_per_application": apply_bytes(V, Nt, prec, degree),
            "peak_source": "%s STREAM-style copy" % peaks_kind}
     hbm["frac"] = hbm["achieved_gbs"] / hbm_peak
     if prec == "fp64":
@@ -771,19 +784,18 @@ def run_ours(args):
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "peak_source": "measured cuBLAS DGEMM 4096^3 on this GPU (FP64 ALU peak)"}
-    elif params.operand_mode == 3:
+    elif params.operand_mode == 3 or degree:
         peak, sms, mhz = fp32_fma_tflops(torch, dev)
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "peak_source": "FP32 FMA rate from unit counts: %d SMs (device attribute) x "
-                               "128 lanes x 2 flop x %.0f MHz (the CUDA-core cluster mode runs "
-                               "on one cluster)" % (sms, mhz)}
+                               "128 lanes x 2 flop x %.0f MHz" % (sms, mhz)}
     else:
         peak = peaks.get("bf16_tflops_sustained", FALLBACK["bf16_tflops_sustained"])
         roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "peak_source": "%s bf16 dense sustained (fp16 has the same rate)" % peaks_kind}
-    roof["flop_per_application"] = flops_per_apply(V, Nt)
+    roof["flop_per_application"] = flops_per_apply(V, Nt, degree)
     roof["applications_per_launch"] = n_app
     roof["traffic_source"] = traffic_src
     roof["hbm"] = hbm
@@ -792,7 +804,7 @@ def run_ours(args):
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": ("f64" if prec == "fp64" else
-                  "f32 (f64 residuals)" if params.operand_mode == 3 else
+                  "f32 (f64 residuals)" if params.operand_mode == 3 or degree else
                   "f16-split/f32 (f64 residuals)"),
         "data": "synthetic",
         "config": {"workload": name, "precision": prec, "L": w["L"], "V": V, "Nt": Nt,
@@ -862,14 +874,14 @@ def run_ours(args):
         dist.destroy_process_group()
 
 
-def apply_bytes(V, Nt, prec):
+def apply_bytes(V, Nt, prec, degree=0):
     """Algorithmic HBM bytes of one application: E once (FP64, or its FP16
-    hi/lo split), the input and output vectors, the phase field phi and the
-    phase table exp(i phi) written and read once."""
+    hi/lo split; nothing for the series), the input and output vectors, the
+    phase field phi and (dense) the phase table exp(i phi) written and read."""
     N = V * Nt
     if prec == "fp64":
-        return 8.0 * V * V + 16.0 * N * 2 + 8.0 * N + 16.0 * N * 2
-    return 4.0 * V * V + 8.0 * N * 2 + 8.0 * N + 8.0 * N * 2
+        return (0.0 if degree else 8.0 * V * V + 32.0 * N) + 16.0 * N * 2 + 8.0 * N
+    return (0.0 if degree else 4.0 * V * V + 16.0 * N) + 8.0 * N * 2 + 8.0 * N
 
 
 def run_apply(args):
@@ -894,10 +906,10 @@ def run_apply(args):
     if args.operand_mode is not None:
         params.operand_mode = args.operand_mode
     elif prec == "mixed" and not args.no_tune:
-        # the standalone tile kinds (site-major 1, slice-major 4, split-K 5),
-        # each timed on a few applications before the timed region
+        # the automatic choice (0: the series) and the standalone tile kinds
+        # (site-major 1, slice-major 4, split-K 5), each timed on a few applications before the timed region
         best = None
-        for mode in (1, 4, 5):
+        for mode in (0, 1, 4, 5):
             try:
                 c = hmc.Context(dataclasses.replace(params, operand_mode=mode))
             except hmc.HmcError:
@@ -967,13 +979,20 @@ def run_apply(args):
         torch, stream, psi, out, lambda: ctx.apply_M(phi, psi, out, prec=p), args.applies)
     n = args.steps * args.applies
     per_ms = total_ms / n
-    flop = flops_per_apply(V, Nt)
-    byts = apply_bytes(V, Nt, prec)
+    degree = series_of(params, prec)
+    flop = flops_per_apply(V, Nt, degree)
+    byts = apply_bytes(V, Nt, prec, degree)
     peaks, kind = load_peaks()
     if prec == "fp64":
         peak = measure_dgemm_tflops(torch)
         roof = {"bound": "alu", "achieved": flop / (per_ms * 1e-3) / 1e12, "peak": peak,
                 "unit": "TFLOP/s", "peak_source": "measured cuBLAS DGEMM 4096^3"}
+    elif degree:
+        peak, sms, mhz = fp32_fma_tflops(torch, dev)
+        roof = {"bound": "alu", "achieved": flop / (per_ms * 1e-3) / 1e12, "peak": peak,
+                "unit": "TFLOP/s",
+                "peak_source": "FP32 FMA rate from unit counts: %d SMs x 128 lanes x 2 flop x "
+                               "%.0f MHz" % (sms, mhz)}
     else:
         peak = peaks.get("bf16_tflops", FALLBACK["bf16_tflops"])
         roof = {"bound": "tensor", "achieved": flop / (per_ms * 1e-3) / 1e12, "peak": peak,
@@ -989,7 +1008,7 @@ def run_apply(args):
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "f64" if prec == "fp64" else "f16-split/f32",
+            "dtype": "f64" if prec == "fp64" else "f32" if degree else "f16-split/f32",
             "data": "synthetic",
             "config": {"workload": name, "mode": "apply", "precision": prec, "V": V, "Nt": Nt,
                        "applies_per_step": args.applies,
@@ -1076,9 +1095,11 @@ def run_cg(args):
     e2e_ms, e2e_in, e2e_out = e2e_host_calls(torch, stream, chi, xbuf, long_solve, 1)
     ms64 = (solve_ms(hmc.PREC_FP64, 2 * n64) - solve_ms(hmc.PREC_FP64, n64)) / n64
     peaks, kind = load_peaks()
-    flop = 2 * flops_per_apply(V, Nt)
-    byts = 2 * apply_bytes(V, Nt, "mixed")
-    peak = peaks.get("bf16_tflops", FALLBACK["bf16_tflops"])
+    degree = series_of(params, "mixed")
+    flop = 2 * flops_per_apply(V, Nt, degree)
+    byts = 2 * apply_bytes(V, Nt, "mixed", degree)
+    peak = fp32_fma_tflops(torch, dev)[0] if degree else \
+        peaks.get("bf16_tflops", FALLBACK["bf16_tflops"])
     hbm_peak = peaks.get("hbm_gbs", FALLBACK["hbm_gbs"])
     achieved = flop / (ms_it * 1e-3) / 1e12
     traffic_it, traffic_src = committed_traffic(name, "per-cg-iteration")
@@ -1086,7 +1107,7 @@ def run_cg(args):
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": statistics.mean(per_it) * (n_long - n_short),
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "f16-split/f32", "data": "synthetic",
+            "dtype": "f32" if degree else "f16-split/f32", "data": "synthetic",
             "config": {"workload": name, "mode": "cg", "V": V, "Nt": Nt,
                        "iterations": [n_short, n_long],
                        "launch_shape": {"team_ctas": params.team_ctas,
@@ -1103,12 +1124,13 @@ def run_cg(args):
                            "memory and x back (its FP64 set-up and final residual "
                            "included, unlike the value)"},
             "gpu_launches": 2 * args.steps,
-            "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak,
-                         "unit": "TFLOP/s", "frac": achieved / peak,
+            "roofline": {"bound": "alu" if degree else "tensor", "achieved": achieved,
+                         "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": (traffic_it * 1.0) if traffic_it is not None else None,
                          "traffic_source": traffic_src,
                          "flop_per_iteration": flop,
-                         "peak_source": "%s bf16 dense burst (fp16 has the same rate)" % kind,
+                         "peak_source": "FP32 FMA rate from unit counts" if degree else
+                         "%s bf16 dense burst (fp16 has the same rate)" % kind,
                          "hbm": {"achieved_gbs": byts / (ms_it * 1e-3) / 1e9,
                                  "peak_gbs": hbm_peak, "algorithmic_bytes": byts,
                                  "frac": byts / (ms_it * 1e-3) / 1e9 / hbm_peak}},
@@ -1285,17 +1307,20 @@ def run_batch(args, emit=True):
         e.synchronize()
         loop_mixed_same_ms = s.elapsed_time(e)
     sizes = [(p.L, p.Nt) for p in plist]
-    flop = sum((applies_per_traj(o, plist[i % n].n_md)) * flops_per_apply(plist[i % n].V,
-                                                                         plist[i % n].Nt)
+    flop = sum(applies_per_traj(o, plist[i % n].n_md) *
+               flops_per_apply(plist[i % n].V, plist[i % n].Nt, series_of(plist[i % n], "mixed"))
                for i, o in enumerate(outs)) / args.steps
     peaks, kind = load_peaks()
-    peak = peaks.get("bf16_tflops_sustained", FALLBACK["bf16_tflops_sustained"])
+    on_series = all(series_of(p, "mixed") for p in plist)
+    peak = fp32_fma_tflops(torch, dev)[0] if on_series else \
+        peaks.get("bf16_tflops_sustained", FALLBACK["bf16_tflops_sustained"])
     achieved = flop / (total_ms / args.steps * 1e-3) / 1e12
     line = {
         "metric": METRIC, "value": value, "unit": "trajectories/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": total_ms / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "f16-split/f32 (f64 residuals)", "data": "synthetic",
+        "dtype": ("f32" if on_series else "f16-split/f32") + " (f64 residuals)",
+        "data": "synthetic",
         "config": {"workload": "batch%d" % n, "precision": "mixed", "chains": n,
                    "L_set": sorted(set(p.L for p in plist)),
                    "Nt_set": sorted(set(p.Nt for p in plist)),
@@ -1328,9 +1353,10 @@ def run_batch(args, emit=True):
                 "h2d_bytes_per_step": e2e_bytes,
                 "d2h_bytes_per_step": e2e_bytes + n * 16 * 8},   # + 16 doubles per chain record
         "gpu_launches": args.steps,
-        "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": None,
-                     "peak_source": "%s bf16 dense sustained (fp16 has the same rate)" % kind},
+        "roofline": {"bound": "alu" if on_series else "tensor", "achieved": achieved,
+                     "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
+                     "peak_source": "FP32 FMA rate from unit counts" if on_series else
+                     "%s bf16 dense sustained (fp16 has the same rate)" % kind},
         "clocks": clk,
     }
     if rank == 0 and world == 1 and not args.no_cpu_baseline:

@@ -6,11 +6,11 @@ not depend on the residual) for candidate shapes -- CTAs of the persistent
 launch (team_ctas), CTAs of the FP32 inner loop (inner_ctas), time slices per
 tensor-core tile (tile_slices), streamed or resident E, site-major or
 slice-major tiles, CUDA-core cluster mode, split-K tiles with E resident
-(operand_mode) -- and keeps the fastest.  Timing uses CUDA
+(operand_mode), the library's automatic choice -- and keeps the fastest.  Timing uses CUDA
 events on the current stream around calls through the C ABI; results are
 cached per (L, Nt, team constraint) for the process.
 """
-import itertools
+import math
 
 import torch
 
@@ -34,6 +34,24 @@ def small_feasible(V, Nt, C):
     total = (r16(V * Vr * 4) + 6 * r16(S * V * 8) + 2 * r16(V * SP * 8) + 2 * r16(V * 8) +
              r16(KS * S * Vr * 8))
     return total <= 208 * 1024
+
+
+def series_degree(rho, tol):
+    """Degree of the polynomial of the sparse hopping that stands for E
+    (csrc/series.h): the Chebyshev tail 2 (rho/2)^(K+1) / (K+1)! below tol
+    e^-rho, rho = 3 |delta kappa|."""
+    K, tail = 0, rho
+    while tail > tol * math.exp(-rho):
+        K += 1
+        tail *= rho / 2 / (K + 1)
+    return K
+
+
+def series_feasible(params):
+    """Host copy of the rule that makes the automatic operand mode (0) the
+    series: rho <= 4, at most 1536 sites, no mass preconditioning."""
+    return 3 * abs(params.delta * params.kappa) <= 4.0 and params.V <= 1536 and \
+        params.L <= 32 and params.hb_inner == 0
 
 
 def team_candidates(params, csize):
@@ -123,6 +141,8 @@ def tune(params, iters=40, reps=2, single_cta=False, seed=1, team=0, modes=None)
         timings = []
         shapes = team_candidates(params, team) if team > 1 else candidates(params, num_sms,
                                                                              single_cta)
+        if not single_cta and team <= 1 and series_feasible(params):
+            shapes = shapes + [(0, 0, 0, 0)]   # the library's automatic choice: the series
         if modes:
             shapes = [sh for sh in shapes if sh[3] in modes]
         for team_c, inner, ns, mode in shapes:
@@ -251,13 +271,18 @@ def plan_teams(est_solo, est_team, num_ctas, csize):
 
 
 def batch_shapes(plist, csize=4, num_sms=None):
-    """Launch shapes of a batch: each chain's tuned one-CTA shape, or a tuned
+    """Launch shapes of a batch: the automatic one where every chain has its
+    series, else each chain's tuned one-CTA shape, or a tuned
     cluster team of csize CTAs for the chains plan_teams picks, each with its
     tuned reliable-update threshold.  The time of a trajectory is estimated
     as the tuned seconds per CG iteration (one CTA, or the team) times Nt (at
     fixed delta the iterations per trajectory grow about in proportion to
     beta = Nt delta); teams are timed only for chains above half the ideal
     makespan."""
+    if all(series_feasible(p) for p in plist):
+        # the series' batch kernel, whose cluster teams the library plans itself
+        return [tune_ru(hmc.Params(**{**p.__dict__, "team_ctas": 0, "inner_ctas": 0,
+                                      "tile_slices": 0, "operand_mode": 0})) for p in plist]
     if num_sms is None:
         dev = torch.device("cuda", torch.cuda.current_device())
         num_sms = torch.cuda.get_device_properties(dev).multi_processor_count
