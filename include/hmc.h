@@ -62,9 +62,10 @@ typedef enum hmc_status {
 
 typedef enum hmc_precision {
     HMC_PREC_FP64 = 0,   /* every step in FP64 on CUDA cores */
-    HMC_PREC_MIXED = 1   /* FP16-split tensor-core contraction, FP32 CG with
-                            FP64 reliable updates; FP64 for residuals, sums,
-                            force and Metropolis */
+    HMC_PREC_MIXED = 1   /* FP32 CG (E by its polynomial in FP32, or as an FP16
+                            split on the tensor cores: hmc_params.operand_mode)
+                            with FP64 reliable updates; FP64 for residuals,
+                            sums, force and Metropolis */
 } hmc_precision;
 
 /* Physics and solver parameters of one Markov chain. */
@@ -93,7 +94,10 @@ typedef struct hmc_params {
                             (operand_mode 4: 1..64; 0: automatic) */
     int inner_ctas;      /* CTAs running the FP32 iterations of the mixed CG
                             (0: automatic; the FP64 steps use all CTAs) */
-    int operand_mode;    /* mixed path: 0 automatic, 1 stream E through shared
+    int operand_mode;    /* mixed path: 0 automatic (E as a polynomial of the
+                            sparse hopping on CTAs that own time slices, where
+                            3 |delta kappa| <= 4, V <= 1536, cluster_mode = 0 and
+                            hb_inner = 0; else tensor-core tiles), 1 stream E through shared
                             memory on every application, 2 keep each CTA's rows
                             of E resident for the whole solve (needs
                             V <= 256 and one CTA per 128-site block; a chain
