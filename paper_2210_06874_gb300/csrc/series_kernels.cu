@@ -201,10 +201,13 @@ int series_ctx_init(hmc_ctx* c) {
         cudaMemset(p, 0, bytes);
         return p;
     };
-    v.ser_mail = (uint64_t*)alloc(2 * T * v.V * 16);
-    v.ser_norm = (uint64_t*)alloc(2 * T * 128);
-    v.ser_seq = (unsigned*)alloc(sizeof(unsigned));
-    if (!v.ser_mail || !v.ser_norm || !v.ser_seq) return HMC_ERR_CUDA;
+    // [mail][norms][sequence number]
+    const size_t mail = 2 * T * v.V * 16, norms = 2 * T * 128;
+    unsigned char* p = (unsigned char*)alloc(mail + norms + 16);
+    if (!p) return HMC_ERR_CUDA;
+    v.ser_mail = (uint64_t*)p;
+    v.ser_norm = (uint64_t*)(p + mail);
+    v.ser_seq = (unsigned*)(p + mail + norms);
     int most = 0;
     if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) !=
         cudaSuccess)

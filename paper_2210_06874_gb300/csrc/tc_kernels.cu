@@ -656,11 +656,12 @@ static void* dev_alloc(hmc_ctx* c, size_t bytes, bool* ok) {
     return p;
 }
 
-int tc_ctx_init(hmc_ctx* c) {
+// The FP16 splits of E, the split-K slots and the tensor maps: what only the
+// tensor-core tiles use.  Contexts on the automatic choice with a series do
+// without (at L = 24 they were most of the context's set-up).
+static int tc_tiles_init(hmc_ctx* c) {
     ChainView& v = c->view;
     const int V = v.V;
-    v.Vr = ((V + tc::TM - 1) / tc::TM) * tc::TM;
-    v.Vp = ((V + tc::KCH - 1) / tc::KCH) * tc::KCH;
     std::vector<double> E((size_t)V * V);
     if (cudaMemcpy(E.data(), v.E, E.size() * sizeof(double), cudaMemcpyDeviceToHost) !=
         cudaSuccess)
@@ -696,21 +697,10 @@ int tc_ctx_init(hmc_ctx* c) {
         }
     v.e_inv = (float)std::ldexp(1.0, -eE);
     bool ok = true;
-    const size_t N = (size_t)v.N;
     void* dhi = dev_alloc(c, hi.size() * sizeof(__half), &ok);
     void* dlo = dev_alloc(c, lo.size() * sizeof(__half), &ok);
     void* dwhi = dev_alloc(c, whi.size() * sizeof(__half), &ok);
     void* dwlo = dev_alloc(c, wlo.size() * sizeof(__half), &ok);
-    v.cis_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    v.r_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    v.p_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    v.p2_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    v.q_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    v.x_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    v.g_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
-    const size_t Nh = (size_t)(v.Nt + 2) * v.V;   // split-K sources with the halo rows
-    v.u_f = (float2*)dev_alloc(c, Nh * sizeof(float2), &ok);
-    v.rh_f = (float2*)dev_alloc(c, Nh * sizeof(float2), &ok);
     v.sk_b16 = nullptr;
     v.sk_maps = nullptr;
     v.gslots = (unsigned long long*)dev_alloc(c, tc::kGatherSlots * sizeof(unsigned long long),
@@ -842,7 +832,28 @@ int tc_ctx_init(hmc_ctx* c) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
             cudaSuccess)
             (void)cudaGetLastError();
-    return series_ctx_init(c);
+    return HMC_OK;
+}
+
+// FP32 workspaces of the mixed path, and what its kernels need.
+int tc_ctx_init(hmc_ctx* c) {
+    ChainView& v = c->view;
+    v.Vr = ((v.V + tc::TM - 1) / tc::TM) * tc::TM;
+    v.Vp = ((v.V + tc::KCH - 1) / tc::KCH) * tc::KCH;
+    bool ok = true;
+    const size_t N = (size_t)v.N;
+    v.cis_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    v.r_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    v.p_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    v.p2_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    v.q_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    v.x_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    v.g_f = (float2*)dev_alloc(c, N * sizeof(float2), &ok);
+    const size_t Nh = (size_t)(v.Nt + 2) * v.V;   // split-K sources with the halo rows
+    v.u_f = (float2*)dev_alloc(c, Nh * sizeof(float2), &ok);
+    v.rh_f = (float2*)dev_alloc(c, Nh * sizeof(float2), &ok);
+    if (!ok) return HMC_ERR_CUDA;
+    return series_chosen(c) ? series_ctx_init(c) : tc_tiles_init(c);
 }
 
 void tc_ctx_free(hmc_ctx* c) {
@@ -1448,7 +1459,12 @@ int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
     std::vector<char> auto_team(n, 0);
     if (b->series) plan_series_teams(b, auto_team);
     std::vector<CUtensorMap> maps(4 * n_maps);
-    for (int i = 0; i < n; ++i)
+    for (int i = 0; i < n && !b->series; ++i)
+        if (!b->ctxs[i]->tc && tc_tiles_init(b->ctxs[i]) != HMC_OK) {
+            tc_batch_destroy(b);
+            return HMC_ERR_CUDA;
+        }
+    for (int i = 0; i < n && !b->series; ++i)
         if (leader[i] == i) {
             maps[4 * map_slot[i]] = b->ctxs[i]->tc->map_hi;
             maps[4 * map_slot[i] + 1] = b->ctxs[i]->tc->map_lo;
@@ -1572,7 +1588,8 @@ int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
                    cudaSuccess))
         ok = false;
     if (ok) {
-        for (int i = 0; i < n; ++i) items[i].maps = b->d_maps + 4 * map_slot[i];
+        for (int i = 0; i < n; ++i)
+            items[i].maps = b->series ? nullptr : b->d_maps + 4 * map_slot[i];
         ok = cudaMemcpy(b->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(),
                         cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(b->d_items, items.data(), sizeof(tc::BatchItem) * n,
