@@ -285,9 +285,10 @@ __device__ inline void cluster_sync_init(ClusterSync* cs, int size) {
 
 // Warp 0 of a cluster team, sync k = cs->count: lane r < size stores this
 // CTA's NV values (FP64 in `part`, or one FP32 in `part_f` when F32) into
-// member r's slot and arrives on member r's barrier k & 1 (release: orders
-// this CTA's earlier writes, shared and global, local and remote, before the
-// arrival).
+// member r's slot and arrives on member r's barrier k & 1.  The arrival's
+// release covers what warp 0 wrote and what a block barrier before the call
+// ordered: team_sync has one on every path, so that all the block's writes,
+// shared and global, local and remote, come before the arrival.
 template <int NV, bool F32>
 __device__ inline void cluster_push(const Team& tm, const double* v, float vf) {
     ClusterSync* cs = tm.cs;
@@ -383,6 +384,9 @@ __device__ inline bool team_sync(Team& tm, double* v) {
         __syncthreads();
         return ok != 0;
     }
+    // the block's writes, and its reads of what the members write next, before
+    // the post of either kind of team (NV > 0: block_reduce or the caller)
+    if constexpr (NV == 0) __syncthreads();
     if (tm.cs) {
         // cluster team: same summation order as the global path below
         // (lane r holds member r's partial, then a fixed shuffle tree)
@@ -415,7 +419,6 @@ __device__ inline bool team_sync(Team& tm, double* v) {
         __syncthreads();
         return ok != 0;
     }
-    if constexpr (NV == 0) __syncthreads();   // the block's writes before the post
     if (threadIdx.x < 32) {
         const unsigned seq = *tm.gen + 1u;
         const bool ok = slot_sync<NV, kF32>(tm, seq, v);

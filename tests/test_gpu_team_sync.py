@@ -1,0 +1,47 @@
+"""The team barrier and sums of csrc/common.cuh between the CTAs of a
+cluster team and of a global-memory team, on the GPU.
+
+* A barrier orders the whole block's writes, not only those of the warp that
+  posts: every warp but the first stores late, and the next CTA reads each word
+  after a plain barrier.  Words and sums are whole numbers, compared exactly.
+"""
+import ctypes
+import os
+import subprocess
+
+import pytest
+import torch
+
+from paper_2210_06874_gb300 import build_lib
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+HERE = os.path.dirname(os.path.abspath(__file__))
+P = ctypes.c_void_p
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("team") / "libteam_sync_probe.so")
+    subprocess.run([build_lib.nvcc(), *build_lib.ARCH, *build_lib.FLAGS, "-shared", "-o", so,
+                    os.path.join(HERE, "team_sync_probe.cu")], check=True)
+    lib = ctypes.CDLL(so)
+    lib.probe_control_bytes.restype = ctypes.c_ulonglong
+    lib.probe_exchange.argtypes = [P, P, P] + [ctypes.c_int] * 4
+    return lib
+
+
+def control(lib):
+    return torch.zeros(lib.probe_control_bytes(), dtype=torch.uint8, device=DEV)
+
+
+@pytest.mark.parametrize("grid,threads,cluster", [(2, 256, 1), (8, 640, 1), (16, 640, 1),
+                                                  (2, 256, 0), (16, 640, 0), (96, 256, 0)])
+def test_barrier_orders_every_warp(probe, grid, threads, cluster):
+    ctl = control(probe)
+    data = torch.zeros(grid * threads, dtype=torch.int32, device=DEV)
+    bad = torch.zeros(1, dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    assert probe.probe_exchange(ctl.data_ptr(), data.data_ptr(), bad.data_ptr(), grid, threads,
+                                200, cluster) == 0
+    assert int(bad) == 0
