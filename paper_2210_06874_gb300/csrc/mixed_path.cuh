@@ -871,12 +871,17 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
 }
 
 // Cluster launch: set up the cluster team state and check that the inner
-// team's ranks are the cluster ranks of cluster 0.
+// team's ranks are the cluster ranks of cluster 0.  A launch that is not made of
+// such clusters ends at its first team sync, which is one of the whole team
+// through global memory: cluster_ok after it, on every thread (the sync orders
+// the status of a member before its post).
 __device__ inline void cluster_begin(const PersistentArgs& pa, ClusterSync* cs, int* status) {
     if (pa.cluster <= 1) return;
-    if (threadIdx.x == 0 && cluster_ctarank() != (uint32_t)(blockIdx.x % pa.cluster))
-        set_status(status, HMC_ERR_UNSUPPORTED);
+    if (threadIdx.x == 0 && !cluster_matches(pa.cluster)) set_status(status, HMC_ERR_UNSUPPORTED);
     cluster_sync_init(cs, pa.cluster);
+}
+__device__ inline bool cluster_ok(const PersistentArgs& pa, const Team& tm) {
+    return pa.cluster <= 1 || !__syncthreads_or(threadIdx.x == 0 && team_failed(tm));
 }
 
 __device__ __forceinline__ Team make_team(const ChainView& c) {
@@ -928,7 +933,7 @@ __device__ bool run_trajectory(const ChainView& c, Team& tm, TcState& st, f64::S
         h0[1] += rho.x * rho.x + rho.y * rho.y;
         h0[2] += zp.x * zp.x;
     }
-    bool ok = team_sum<3>(tm, h0);
+    bool ok = team_sum<3>(tm, h0) && cluster_ok(pa, tm);
     const double H0 = 0.5 * h0[0] * inv_dU + h0[1] + 0.5 * h0[2];
     f64::EpiArgs ea = {};
     if (ok) {
@@ -1101,6 +1106,14 @@ __device__ inline void batch_loop(const BatchItem* __restrict__ items,
                                   const BatchCallArgs* call, double* outs, int csize,
                                   ClusterSync* cs, Run&& run) {
     __shared__ int s_idx;
+    if (csize > 1 && !cluster_matches(csize)) {
+        // launched without its clusters (every CTA alike): no chain runs
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+            outs[(size_t)i * kNumScalars + kTrajSolves] = 0.0;
+            outs[(size_t)i * kNumScalars + kTrajStatus] = (double)HMC_ERR_UNSUPPORTED;
+        }
+        return;
+    }
     const int crank = csize > 1 ? (int)cluster_ctarank() : 0;
     bool solo = csize == 1;
     bool ok = true;

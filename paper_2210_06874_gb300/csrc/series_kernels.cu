@@ -63,9 +63,9 @@ struct Launch {
     int cluster;        // the grid is one cluster of this many CTAs (0: global team)
     unsigned smem;      // dynamic shared memory in bytes
 };
-__device__ __forceinline__ Team begin(const ChainView& c, const Launch& la, ClusterSync* cs,
-                                      uint64_t* norm, unsigned* seq, Work& wk) {
-    Team tm = tc::make_team(c);
+__device__ __forceinline__ bool begin(const ChainView& c, const Launch& la, ClusterSync* cs,
+                                      uint64_t* norm, unsigned* seq, Work& wk, Team& tm) {
+    tm = tc::make_team(c);
     wk.bytes = la.smem;
     wk.mail_V = la.cluster ? c.V : 0;
     wk.norm_smem = norm;
@@ -75,12 +75,16 @@ __device__ __forceinline__ Team begin(const ChainView& c, const Launch& la, Clus
         uint64_t* m = reinterpret_cast<uint64_t*>(ser_dyn);
         for (int i = threadIdx.x; i < (int)(mail_bytes(c.V) / 8); i += blockDim.x) m[i] = 0;
         if (threadIdx.x < 32) norm[threadIdx.x] = 0;
+        if (threadIdx.x == 0 &&
+            !(cluster_matches(la.cluster) && gridDim.x == (unsigned)la.cluster))
+            set_status(c.status, HMC_ERR_UNSUPPORTED);
         __syncthreads();
         cluster_sync_init(cs, la.cluster);
+        if (__syncthreads_or(threadIdx.x == 0 && team_failed(tm))) return false;
         tm.cs = cs;
     }
     __syncthreads();
-    return tm;
+    return true;
 }
 // No member leaves while others may still write to it; the context's next
 // launch starts past every number any CTA can have used.
@@ -96,7 +100,8 @@ __device__ __forceinline__ void end(const ChainView& c, const Launch& la, const 
     __shared__ uint64_t s_norm[32];                                                       \
     __shared__ unsigned s_seq;                                                            \
     Work wk;                                                                              \
-    Team tm = begin(c, la, &s_cs, s_norm, &s_seq, wk);                                    \
+    Team tm;                                                                              \
+    if (!begin(c, la, &s_cs, s_norm, &s_seq, wk, tm)) return;                             \
     tc::TcState st;                                                                       \
     st.ser = &wk
 

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(NTHR, 1)
     cluster_begin(pa, &s_cs, c.status);
     set_phases(c, tm, phi);
     MixedResult res{};
-    bool ok = team_barrier(tm);
+    bool ok = team_barrier(tm) && cluster_ok(pa, tm);
     if (ok) ok = cg_mixed<KIND>(c, tm, st, sm64, &mhi, &mlo, pa, &s_cs, chi, x, res);
     if (ok && tm.rank == 0 && threadIdx.x == 0) {
         c.scalars[0] = res.iterations;
@@ -388,7 +388,7 @@ __device__ __noinline__ bool run_trajectory_hb(const ChainView& c, Team& tm, TcS
         h0[1] += r1.x * r1.x + r1.y * r1.y + r2.x * r2.x + r2.y * r2.y;
         h0[2] += zp.x * zp.x;
     }
-    if (!team_sum<3>(tm, h0)) return false;
+    if (!team_sum<3>(tm, h0) || !cluster_ok(pa, tm)) return false;
     const double H0 = 0.5 * h0[0] * inv_dU + h0[1] + 0.5 * h0[2];
     int iters_in = 0, iters_out = 0, solves_in = 0, solves_out = 0, rus = 0, fp64_iters = 0;
     int status = HMC_OK;

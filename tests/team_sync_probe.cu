@@ -49,7 +49,57 @@ __global__ void k_exchange(ChainView c, unsigned* data, int rounds, int cluster,
     if (cluster) cluster_barrier_all();
 }
 
+// One CTA sets the status word before its third sync: res[rank] = the syncs
+// that succeeded before one failed (kind 0: plain barriers, 1: sums of three
+// values, 2: FP32 sums).
+__global__ void k_status(ChainView c, int setter, int kind, int* res) {
+    __shared__ unsigned gen;
+    Team tm = probe_team(c, nullptr, &gen, false);
+    int good = 0;
+    for (; good < 8; ++good) {
+        if (good == 2 && tm.rank == setter && threadIdx.x == 0)
+            set_status(tm.status, HMC_ERR_UNSUPPORTED);
+        double v[3] = {1.0, 2.0, 3.0};
+        float f = 0.f;
+        const bool ok = kind == 0   ? team_barrier(tm)
+                        : kind == 1 ? team_sum<3>(tm, v)
+                                    : team_sum_f(tm, 1.f, f);
+        if (!ok) break;
+    }
+    if (threadIdx.x == 0) res[tm.rank] = good;
+}
+
+// res[CTA] = what cluster_matches says of a launch in clusters of `size`.
+__global__ void k_matches(int size, int* res) {
+    if (threadIdx.x == 0) res[blockIdx.x] = cluster_matches(size) ? 1 : 0;
+}
+
 }  // namespace
+
+extern "C" int probe_status(void* control, int* res, int grid, int threads, int setter, int kind) {
+    ChainView c{};
+    control_bind(&c, control);
+    void* args[] = {&c, &setter, &kind, &res};
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_status, dim3(grid), dim3(threads),
+                                                args, 0, nullptr);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    return (int)e;
+}
+
+extern "C" int probe_matches(int* res, int grid, int launched, int size) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(32);
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeClusterDimension;
+    a[0].val.clusterDim.x = (unsigned)launched;
+    a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+    cfg.attrs = a;
+    cfg.numAttrs = launched > 0 ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_matches, size, res);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    return (int)e;
+}
 
 // Control block (zeroed), words (zeroed) and counter are the caller's device memory.
 extern "C" int probe_exchange(void* control, unsigned* data, int* bad, int grid, int threads,

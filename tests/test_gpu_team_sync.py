@@ -4,6 +4,9 @@ cluster team and of a global-memory team, on the GPU.
 * A barrier orders the whole block's writes, not only those of the warp that
   posts: every warp but the first stores late, and the next CTA reads each word
   after a plain barrier.  Words and sums are whole numbers, compared exactly.
+* A status word that one CTA sets before its post ends the team on every CTA at
+  that sync or the next one, even when all of them arrive.
+* What tells such a launch: cluster_matches.
 """
 import ctypes
 import os
@@ -28,6 +31,8 @@ def probe(tmp_path_factory):
     lib = ctypes.CDLL(so)
     lib.probe_control_bytes.restype = ctypes.c_ulonglong
     lib.probe_exchange.argtypes = [P, P, P] + [ctypes.c_int] * 4
+    lib.probe_status.argtypes = [P, P] + [ctypes.c_int] * 4
+    lib.probe_matches.argtypes = [P] + [ctypes.c_int] * 3
     return lib
 
 
@@ -45,3 +50,22 @@ def test_barrier_orders_every_warp(probe, grid, threads, cluster):
     assert probe.probe_exchange(ctl.data_ptr(), data.data_ptr(), bad.data_ptr(), grid, threads,
                                 200, cluster) == 0
     assert int(bad) == 0
+
+
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("grid,setter", [(2, 1), (33, 0), (96, 95)])
+def test_status_ends_the_sync(probe, grid, setter, kind):
+    ctl = control(probe)
+    res = torch.full((grid,), -1, dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    assert probe.probe_status(ctl.data_ptr(), res.data_ptr(), grid, 256, setter, kind) == 0
+    assert set(res.tolist()) <= {2, 3}          # of 8 syncs
+
+
+@pytest.mark.parametrize("grid,launched,size,want", [(8, 4, 4, 1), (8, 8, 8, 1), (8, 4, 2, 0),
+                                                     (8, 2, 4, 0), (8, 0, 2, 0), (8, 0, 1, 1)])
+def test_launch_without_its_clusters_is_told(probe, grid, launched, size, want):
+    res = torch.full((grid,), -1, dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    assert probe.probe_matches(res.data_ptr(), grid, launched, size) == 0
+    assert res.tolist() == [want] * grid
