@@ -403,6 +403,12 @@ int hmc_debug_team_padding(hmc_ctx* c, int extra_ctas) {
     return HMC_OK;
 }
 
+int hmc_debug_withhold(hmc_ctx* c, int what) {
+    if (!c || what < 0 || what > 7) return HMC_ERR_BAD_ARG;
+    c->view.withhold = what;
+    return HMC_OK;
+}
+
 int hmc_rng_draw(uint64_t seed, uint32_t stream_id, uint64_t traj, uint32_t chain, int64_t n,
                  uint32_t* raw, double* z0, double* z1, void* stream) {
     if (n < 0 || n > (1LL << 32)) return HMC_ERR_BAD_ARG;

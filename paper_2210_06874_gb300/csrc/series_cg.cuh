@@ -89,6 +89,7 @@ __device__ __forceinline__ uint32_t peer(uint32_t addr, int rank) {
 
 struct Link {
     int T, rank;
+    int posts;          // members that get this CTA's norms: T (0: withheld, testing)
     bool cluster;
     // mail boxes of this CTA's receivers and its own, per kind: cell c's two
     // 16-byte words at 32 c (shared-memory addresses in a cluster, else global)
@@ -97,14 +98,19 @@ struct Link {
     uint64_t* norm;    // [2 kinds][T] every 16 words (global) or [2][16] (own shared memory)
 
     // msg: [2 kinds][T][V] x 2 words (global) or [2][mail_V] x 2 (shared memory)
+    // withhold (see ChainView): rank 0's norms go nowhere, a boundary slice into its
+    // own box instead of its neighbour's, so that every wait for them runs out
     __device__ __forceinline__ void init(const Team& tm, int V, int mail_V, uint64_t* msg,
-                                         uint64_t* nrm) {
+                                         uint64_t* nrm, int withhold) {
         T = tm.size;
         rank = tm.rank;
+        const int held = rank == 0 ? withhold : 0;
+        posts = (held & 1) ? 0 : T;
         cluster = tm.cs != nullptr;
         norm = nrm;
-        const int dst[2] = {rank == 0 ? T - 1 : rank - 1, rank == T - 1 ? 0 : rank + 1};
+        int dst[2] = {rank == 0 ? T - 1 : rank - 1, rank == T - 1 ? 0 : rank + 1};
         for (int k = 0; k < 2; ++k) {
+            if (held & (2 << k)) dst[k] = rank;
             if (cluster) {
                 own_s[k] = cta_smem_u32(msg) + 16u * (uint32_t)(k * mail_V);
                 to_s[k] = peer(own_s[k], dst[k]);
@@ -157,12 +163,12 @@ struct Link {
         const int lane = threadIdx.x & 31;
         const uint64_t w = tagged(v, seq);
         if (cluster) {
-            if (lane < T)
+            if (lane < posts)
                 asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(
                                  peer(cta_smem_u32(norm + kind * 16 + rank), lane)),
                              "l"(w)
                              : "memory");
-        } else if (lane == 0) {
+        } else if (lane == 0 && posts > 0) {
             asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
                              norm + ((size_t)kind * T + rank) * 16),
                          "l"(w)
@@ -434,9 +440,10 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
         g.max_iter = max_iter;
         g.status = tm.status;
         if (tm.cs)
-            g.lk.init(tm, c.V, wk.mail_V, reinterpret_cast<uint64_t*>(ser_dyn), wk.norm_smem);
+            g.lk.init(tm, c.V, wk.mail_V, reinterpret_cast<uint64_t*>(ser_dyn), wk.norm_smem,
+                      c.withhold);
         else
-            g.lk.init(tm, c.V, 0, c.ser_mail, c.ser_norm);
+            g.lk.init(tm, c.V, 0, c.ser_mail, c.ser_norm, c.withhold);
     }
     if (threadIdx.x < kSerMax32) s_ratio[threadIdx.x] = c.ser.r32[threadIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nww = (blockDim.x >> 5) - 1;
