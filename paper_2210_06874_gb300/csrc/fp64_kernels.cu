@@ -101,9 +101,17 @@ __global__ void k_sum_partials(const double* __restrict__ partials, int n, doubl
     if (threadIdx.x == 0) *out = v[0];
 }
 
+// Least CTAs per SM of the persistent kernels.  Left alone, the compiler takes 64
+// registers for the dense form and spills: 15.48 ms for an L = 3, Nt = 8
+// trajectory against 15.24 with the 106 that two CTAs leave it (15.31-15.37 with
+// 80 for three), and 688 against 681 us per CG iteration at L = 33, Nt = 8.
+// 0: the compiler's choice.
+template <int FORM>
+constexpr int kMinCtas = FORM == FORM_DENSE ? 2 : 0;
+
 // scalars: [0] iterations [1] true residual [2] status
 template <int FORM>
-__global__ void __launch_bounds__(NTHR) k_cg(const __grid_constant__ ChainView c, const double* phi, const double2* chi,
+__global__ void __launch_bounds__(NTHR, kMinCtas<FORM>) k_cg(const __grid_constant__ ChainView c, const double* phi, const double2* chi,
                                              double2* x, double tol, int max_iter) {
     __shared__ Smem sm;
     Team tm = make_team(c);
@@ -120,7 +128,7 @@ __global__ void __launch_bounds__(NTHR) k_cg(const __grid_constant__ ChainView c
 
 // scalars: see TrajSlot in launch.h
 template <int FORM>
-__global__ void __launch_bounds__(NTHR) k_trajectory(const __grid_constant__ ChainView c, TrajArgs a) {
+__global__ void __launch_bounds__(NTHR, kMinCtas<FORM>) k_trajectory(const __grid_constant__ ChainView c, TrajArgs a) {
     __shared__ Smem sm;
     Team tm = make_team(c);
     double* phi = a.phi;
@@ -225,7 +233,7 @@ __global__ void __launch_bounds__(NTHR) k_trajectory(const __grid_constant__ Cha
 // Consecutive inner kicks are merged.  Every solve starts from zero.
 // Scalars as k_trajectory, plus the outer level's CG iterations and solves.
 template <int FORM>
-__global__ void __launch_bounds__(NTHR) k_trajectory_hb(const __grid_constant__ ChainView c, TrajArgs a) {
+__global__ void __launch_bounds__(NTHR, kMinCtas<FORM>) k_trajectory_hb(const __grid_constant__ ChainView c, TrajArgs a) {
     __shared__ Smem sm;
     Team tm = make_team(c);
     double* phi = a.phi;
