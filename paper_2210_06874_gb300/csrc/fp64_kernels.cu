@@ -412,7 +412,7 @@ static int series_threads(const ChainView& c) {
 
 int launch_apply_f64(const ChainView& c, bool dag, const double* phi, const double2* in,
                      double2* out, cudaStream_t s) {
-    if (f64::series_form(c, c.V)) {
+    if (f64::series_form(c, false)) {
         const int thr = series_threads(c);
         const size_t sm = (size_t)c.V * sizeof(double);
         if (dag)
@@ -432,7 +432,7 @@ int launch_apply_f64(const ChainView& c, bool dag, const double* phi, const doub
 
 int launch_force_f64(const ChainView& c, const double* phi, const double2* x, double* F,
                      cudaStream_t s) {
-    if (f64::series_form(c, c.V)) {
+    if (f64::series_form(c, false)) {
         f64::k_force_series<<<c.Nt, series_threads(c), (size_t)c.V * sizeof(double), s>>>(
             c, phi, x, F);
         return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
@@ -445,7 +445,7 @@ int launch_force_f64(const ChainView& c, const double* phi, const double2* x, do
 
 // CTAs worth launching for the tiles of one application.
 static int f64_tiles(const ChainView& c) {
-    return f64::series_form(c, f64::kHopDoubles) ? c.Nt : dense_tiles(c);
+    return f64::series_form(c, true) ? c.Nt : dense_tiles(c);
 }
 
 int launch_action(const ChainView& c, const double* phi, const double2* chi, const double2* x,
@@ -461,7 +461,7 @@ int launch_action(const ChainView& c, const double* phi, const double2* chi, con
 
 int launch_cg_f64(const ChainView& c, int num_sms, const double* phi, const double2* chi,
                   double2* x, double tol, int max_iter, cudaStream_t s) {
-    const void* fn = f64::series_form(c, f64::kHopDoubles)
+    const void* fn = f64::series_form(c, true)
                          ? (const void*)f64::k_cg<f64::FORM_SERIES>
                          : (const void*)f64::k_cg<f64::FORM_DENSE>;
     const int grid = persistent_grid(fn, f64::NTHR, num_sms, f64_tiles(c));
@@ -474,7 +474,7 @@ int launch_cg_f64(const ChainView& c, int num_sms, const double* phi, const doub
 }
 
 int launch_trajectory_f64(const ChainView& c, int num_sms, const TrajArgs& a, cudaStream_t s) {
-    const bool ser = f64::series_form(c, f64::kHopDoubles);
+    const bool ser = f64::series_form(c, true);
     const void* fn = a.hb_inner > 0
                          ? (ser ? (const void*)f64::k_trajectory_hb<f64::FORM_SERIES>
                                 : (const void*)f64::k_trajectory_hb<f64::FORM_DENSE>)

@@ -15,9 +15,10 @@
 //           sites in chunks of KC.  E is symmetric, so the chunk
 //           E[i0.., k0..] is read as rows k of E (coalesced) and stored
 //           k-major in shared memory.
-// The series is used where it exists (c.ser.ok), its hop buffer fits and
-// V > 32 (series_form); the dense form serves small lattices, an E given from
-// outside, 3 |delta kappa| > 4 and L > 27 (persistent kernels) or 32.
+// The series is used where it exists (c.ser.ok), its hop buffer fits and it pays
+// (series_form); the dense form serves small lattices, an E given from
+// outside, 3 |delta kappa| > 4 (at L = 5 and 6 from degree 14 or 20 on) and
+// L > 27 (persistent kernels) or 32.
 // Measured, one application / one CG iteration, dense -> series: L = 6,
 // Nt = 32 18.3 -> 10.7 us / 41.6 -> 25.7 us; L = 12, Nt = 64 46.3 -> 13.8 /
 // 95.8 -> 31; L = 24, Nt = 96 477 -> 38 / 940 -> 71; but L = 3, Nt = 8 8.1 ->
@@ -220,8 +221,10 @@ __device__ __forceinline__ void hop_horner(const HopSeries& hs, const Cells<NC>&
     }
 }
 
-__host__ __device__ inline bool series_form(const ChainView& c, int doubles) {
-    return c.ser.ok && c.V > 32 && c.V <= doubles;
+// solve: in a persistent kernel, on the hop buffer of its shared operands; else a
+// standalone application, whose buffer has the slice's size.
+__host__ __device__ inline bool series_form(const ChainView& c, bool solve) {
+    return c.ser.ok && series_pays64(c.V, c.ser.k64, solve) && (!solve || c.V <= kHopDoubles);
 }
 
 // Slices per series tile on a hop buffer of `doubles`: enough to give every
@@ -379,7 +382,7 @@ __device__ __forceinline__ double dense_team(const ChainView& c, const Team& tm,
 template <int FORM, bool DAG, int EPI>
 __device__ __noinline__ double series_team(const ChainView& c, const Team tm, const double2* in,
                                            double2* out, const EpiArgs& ea, Smem& sm) {
-    if (FORM == FORM_EITHER && !series_form(c, kHopDoubles))
+    if (FORM == FORM_EITHER && !series_form(c, true))
         return dense_team<DAG, EPI>(c, tm, in, out, ea, sm);
     double acc = 0.0;
     // (V <= kHopDoubles: at most 768 cells; 256 threads, or at least half of

@@ -13,6 +13,12 @@
 
 #include <math.h>
 
+#ifdef __CUDACC__
+#define HMC_HD __host__ __device__
+#else
+#define HMC_HD
+#endif
+
 namespace hmc {
 
 constexpr int kSerMax64 = 40;   // largest degree kept (FP64)
@@ -32,6 +38,20 @@ struct HopSeries {
 // largest L (4 cells per thread of a 256-thread block).
 constexpr double kSerMaxRho = 4.0;
 constexpr int kSerMaxL = 32;
+
+// Whether the FP64 series beats the dense form, whose tiles pad V to chunks of 32
+// sites: 6 k64 FP64 instructions per site, in 2 k64 steps that wait for one
+// another, against 64 per chunk.  Dense / series, microseconds per CG iteration:
+//   L = 5 (2 chunks)  29.8 / 28.8 at degree 11, 32.7 at 14, 36.7 at 17
+//   L = 6 (3)         39.3 / 28.5 at 11, 36.3 at 17, 41.6 at 21, 46.9 at 25
+//   L = 7 (4)         53.0 / 29.0 at 11, 47.0 at 25
+// and of one application, which the dense form does in two launches:
+//   L = 5             16.5 / 14.4 at 14, 16.5 at 17, 18.5 at 21
+//   L = 6             20.6 / 16.5 at 17, 18.5 at 21, 20.5 at 23
+// Up to 32 sites a slice fills a third of a warp and the dense form is ahead.
+HMC_HD inline bool series_pays64(int V, int k64, bool solve) {
+    return V > 32 && 2 * k64 <= (solve ? 13 : 14) * ((V + 31) / 32);
+}
 
 // Economised power series of exp(rho t) on |t| <= 1: from the Taylor
 // coefficients rho^m / m!, each power t^m above the degree is replaced by its
