@@ -8,7 +8,8 @@ tensor-core tile (tile_slices), streamed or resident E, site-major or
 slice-major tiles, CUDA-core cluster mode, split-K tiles with E resident
 (operand_mode), the library's automatic choice -- and keeps the fastest.  Timing uses CUDA
 events on the current stream around calls through the C ABI; results are
-cached per (L, Nt, team constraint) for the process.
+cached for the process per lattice, delta, team constraint and whether the
+automatic choice is the series.
 """
 import math
 
@@ -49,9 +50,14 @@ def series_degree(rho, tol):
 
 def series_feasible(params):
     """Host copy of the rule that makes the automatic operand mode (0) the
-    series: rho <= 4, at most 1536 sites, no mass preconditioning."""
+    series: rho <= 4, at most 1536 sites, no mass preconditioning, cluster_mode 0."""
     return 3 * abs(params.delta * params.kappa) <= 4.0 and params.V <= 1536 and \
-        params.L <= 32 and params.hb_inner == 0
+        params.L <= 32 and params.hb_inner == 0 and params.cluster_mode == 0
+
+
+def _tune_key(params, single_cta, team, modes):
+    return (params.L, params.Nt, round(params.beta / params.Nt, 12), single_cta, team,
+            tuple(modes) if modes else None, series_feasible(params))
 
 
 def team_candidates(params, csize):
@@ -126,8 +132,7 @@ def tune(params, iters=40, reps=2, single_cta=False, seed=1, team=0, modes=None)
     operand_mode set to the fastest measured shape (team > 1: among the
     shapes of a cluster team of that many CTAs; modes: only those operand
     modes, e.g. (5,) for mass preconditioning on the mixed path)."""
-    key = (params.L, params.Nt, round(params.beta / params.Nt, 12), single_cta, team,
-           tuple(modes) if modes else None)
+    key = _tune_key(params, single_cta, team, modes)
     if key in _cache:
         (team_c, inner, ns, mode), _ = _cache[key]
     else:
@@ -185,7 +190,8 @@ def tune_ru(params, candidates=(0.003, 0.01, 0.05, 0.2), seed=2):
     FP64 updates pay where the FP64 work runs on few CTAs, frequent ones
     where the FP32 iteration stalls early)."""
     key = (params.L, params.Nt, round(params.beta / params.Nt, 12), params.team_ctas,
-           params.inner_ctas, params.tile_slices, params.operand_mode, params.cg_tol)
+           params.inner_ctas, params.tile_slices, params.operand_mode, params.cg_tol,
+           series_feasible(params))
     if key not in _ru_cache:
         dev = torch.device("cuda", torch.cuda.current_device())
         g = torch.Generator(device="cpu").manual_seed(seed)
@@ -216,8 +222,7 @@ def tune_ru(params, candidates=(0.003, 0.01, 0.05, 0.2), seed=2):
 def seconds_per_iteration(params, single_cta=False, team=0):
     """Measured seconds per CG iteration of the shape tune() chose."""
     tune(params, single_cta=single_cta, team=team)
-    key = (params.L, params.Nt, round(params.beta / params.Nt, 12), single_cta, team, None)
-    return _cache[key][1]
+    return _cache[_tune_key(params, single_cta, team, None)][1]
 
 
 def simulate_batch(est_solo, est_team, is_team, num_ctas, csize):
