@@ -12,6 +12,7 @@
 #pragma once
 
 #include <math.h>
+#include <stddef.h>
 
 #ifdef __CUDACC__
 #define HMC_HD __host__ __device__
@@ -51,6 +52,13 @@ constexpr int kSerMaxL = 32;
 // Up to 32 sites a slice fills a third of a warp and the dense form is ahead.
 HMC_HD inline bool series_pays64(int V, int k64, bool solve) {
     return V > 32 && 2 * k64 <= (solve ? 13 : 14) * ((V + 31) / 32);
+}
+
+// Whether a CG vector of S slices of V sites (8 bytes each) still fits a shared
+// memory of `bytes` whose first `top` are taken.  In 64 bits: one CTA may own 2^30
+// site-slices.
+HMC_HD inline bool vector_fits(size_t top, int S, int V, size_t bytes) {
+    return top + (size_t)S * (size_t)V * 8 <= bytes;
 }
 
 // Economised power series of exp(rho t) on |t| <= 1: from the Taylor

@@ -478,10 +478,10 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
     uint32_t top = (uint32_t)mail_bytes(wk.mail_V);
     float4* const hopbuf = reinterpret_cast<float4*>(ser_dyn + top);
     top += (uint32_t)hop_bytes(c.V, sh);
-    const uint32_t vec = (uint32_t)(sh.S * c.V * sizeof(float2));
+    const uint32_t vec = (uint32_t)(sh.S * c.V * sizeof(float2));   // (of one that fits)
     Vec<ST> r, p, G, q, cis, x, Z;
     auto take = [&](auto& v, float2* fallback) {
-        if (ST != kAny || top + vec <= wk.bytes) {
+        if (ST != kAny || vector_fits(top, sh.S, c.V, wk.bytes)) {
             v.off = top;
             v.m = reinterpret_cast<float4*>(ser_dyn + top);
             top += vec;
