@@ -89,7 +89,6 @@ __device__ __forceinline__ uint32_t peer(uint32_t addr, int rank) {
 
 struct Link {
     int T, rank;
-    int posts;          // members that get this CTA's norms: T (0: withheld, testing)
     bool cluster;
     // mail boxes of this CTA's receivers and its own, per kind: cell c's two
     // 16-byte words at 32 c (shared-memory addresses in a cluster, else global)
@@ -98,19 +97,17 @@ struct Link {
     uint64_t* norm;    // [2 kinds][T] every 16 words (global) or [2][16] (own shared memory)
 
     // msg: [2 kinds][T][V] x 2 words (global) or [2][mail_V] x 2 (shared memory)
-    // withhold (see ChainView): rank 0's norms go nowhere, a boundary slice into its
-    // own box instead of its neighbour's, so that every wait for them runs out
+    // withhold (see ChainView): a boundary slice of rank 0 goes into its own box
+    // instead of its neighbour's
     __device__ __forceinline__ void init(const Team& tm, int V, int mail_V, uint64_t* msg,
                                          uint64_t* nrm, int withhold) {
         T = tm.size;
         rank = tm.rank;
-        const int held = rank == 0 ? withhold : 0;
-        posts = (held & 1) ? 0 : T;
         cluster = tm.cs != nullptr;
         norm = nrm;
         int dst[2] = {rank == 0 ? T - 1 : rank - 1, rank == T - 1 ? 0 : rank + 1};
         for (int k = 0; k < 2; ++k) {
-            if (held & (2 << k)) dst[k] = rank;
+            if (rank == 0 && (withhold & (2 << k))) dst[k] = rank;
             if (cluster) {
                 own_s[k] = cta_smem_u32(msg) + 16u * (uint32_t)(k * mail_V);
                 to_s[k] = peer(own_s[k], dst[k]);
@@ -163,12 +160,12 @@ struct Link {
         const int lane = threadIdx.x & 31;
         const uint64_t w = tagged(v, seq);
         if (cluster) {
-            if (lane < posts)
+            if (lane < T)
                 asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(
                                  peer(cta_smem_u32(norm + kind * 16 + rank), lane)),
                              "l"(w)
                              : "memory");
-        } else if (lane == 0 && posts > 0) {
+        } else if (lane == 0) {
             asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
                              norm + ((size_t)kind * T + rank) * 16),
                          "l"(w)
@@ -383,7 +380,7 @@ struct Work {
 // The loop invariants of a segment (shared memory).
 struct Geo {
     int LL, Nt, S, t0, SB, stride, K, it_end, max_iter;
-    bool alone;
+    bool alone, posts;   // posts: the team gets this CTA's norms (see ChainView::withhold)
     float c0, rmax, stop, ru2;
     size_t g0;      // first element of the own slices in [Nt][V]
     int* status;
@@ -426,6 +423,7 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
         g.LL = c.V / 2;
         g.Nt = c.Nt;
         g.alone = tm.size == 1;
+        g.posts = !g.alone && !(tm.rank == 0 && (c.withhold & 1));
         g.t0 = t_lo(tm.rank, c.Nt, tm.size);
         g.S = t_lo(tm.rank + 1, c.Nt, tm.size) - g.t0;
         g.SB = min(sh.SB, g.S);
@@ -550,7 +548,7 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
                 own = __shfl_sync(0xffffffffu, a, 0);
-                if (!g.alone) g.lk.post(kind, own, seq);
+                if (g.posts) g.lk.post(kind, own, seq);
             });
 #pragma unroll
             for (int j = 0; j < N; ++j)
