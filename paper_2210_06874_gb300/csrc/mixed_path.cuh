@@ -536,8 +536,8 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
                          const PersistentArgs& pa, ClusterSync* ics, const double2* chi,
                          double2* x64, MixedResult& res, bool warm = false, double gm1 = 0.0) {
     // the heavy operator M_g of mass preconditioning (gm1 = g - 1 != 0) is
-    // built into the split-K tiles' and the series' epilogues only
-    if (gm1 != 0.0 && KIND != kKindSplitK && KIND != kKindSeries) {
+    // built into the split-K tiles' epilogues only
+    if (gm1 != 0.0 && KIND != kKindSplitK) {
         set_status(tm.status, HMC_ERR_UNSUPPORTED);
         return false;
     }
@@ -695,7 +695,7 @@ __device__ bool cg_mixed(const ChainView& c, Team& tm, TcState& st, f64::Smem& s
         if constexpr (KIND == kKindSeries) {
             const int reason =
                 ser::run_segment(c, ti, *static_cast<const ser::Work*>(st.ser), s_cg, refresh,
-                                 pa.max_iter, x64, (float)(1.0 + gm1));
+                                 pa.max_iter, x64);
             if (reason < 0) return false;
             refresh = false;
             if (tm.rank == 0 && threadIdx.x == 0) {

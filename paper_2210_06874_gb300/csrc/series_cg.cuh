@@ -407,7 +407,7 @@ __host__ __device__ inline size_t shared_bytes(int V, int mail_V, const Shape& s
 template <int ST, int N>
 __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Work& wk,
                                     const Shape sh, tc::CgScalars& s_cg, bool refresh,
-                                    int max_iter, double2* x64, float hop_scale) {
+                                    int max_iter, double2* x64) {
     if (cta_smem_u32(ser_dyn) & 15u) {   // (the mail's 16-byte accesses)
         set_status(tm.status, HMC_ERR_UNSUPPORTED);
         return -1;
@@ -430,7 +430,7 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
         g.stride = sh.SB * g.LL;
         g.g0 = (size_t)g.t0 * c.V;
         g.K = c.ser.k32;
-        g.c0 = c.ser.c0f * hop_scale;
+        g.c0 = c.ser.c0f;
         g.rmax = s_cg.rmax;
         g.stop = s_cg.stop;
         g.ru2 = s_cg.ru2;
@@ -647,14 +647,14 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
 }
 
 __device__ inline int run_segment(const ChainView& c, const Team& tm, const Work& wk,
-                                  tc::CgScalars& s_cg, bool refresh, int max_iter, double2* x64,
-                                  float hop_scale) {
+                                  tc::CgScalars& s_cg, bool refresh, int max_iter,
+                                  double2* x64) {
     const Shape sh = shape(c.L, c.Nt, tm.size);
     if (shared_bytes(c.V, wk.mail_V, sh, kVecs + 1) > wk.bytes)
-        return segment<kAny, 2>(c, tm, wk, sh, s_cg, refresh, max_iter, x64, hop_scale);
+        return segment<kAny, 2>(c, tm, wk, sh, s_cg, refresh, max_iter, x64);
     if (sh.N == 1)
-        return segment<kShared, 1>(c, tm, wk, sh, s_cg, refresh, max_iter, x64, hop_scale);
-    return segment<kShared, 2>(c, tm, wk, sh, s_cg, refresh, max_iter, x64, hop_scale);
+        return segment<kShared, 1>(c, tm, wk, sh, s_cg, refresh, max_iter, x64);
+    return segment<kShared, 2>(c, tm, wk, sh, s_cg, refresh, max_iter, x64);
 }
 
 }  // namespace ser

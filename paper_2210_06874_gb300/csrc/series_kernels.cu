@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 }  // namespace ser
 
 // ---------------------------------------------------------------- host side
-const void* series_batch_kernel(unsigned* smem) {
+const void* series_batch_kernel(unsigned* smem, int* threads) {
+    *threads = ser::kThreads;
     const void* k = (const void*)ser::k_batch;
     int dev = 0, most = 0;
     cudaFuncAttributes at;

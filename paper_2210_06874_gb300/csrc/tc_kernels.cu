@@ -1449,8 +1449,7 @@ int tc_batch_create(const hmc_params* p, int n, TcBatch** out) {
     b->threads = tc::NTHR;
     b->smem = (unsigned)tc::kSmemBytes;
     if (b->series) {
-        b->kernel = series_batch_kernel(&b->smem);
-        b->threads = kSeriesThreads;
+        b->kernel = series_batch_kernel(&b->smem, &b->threads);
         if (!b->kernel) {
             tc_batch_destroy(b);
             return HMC_ERR_CUDA;

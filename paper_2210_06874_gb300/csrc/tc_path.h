@@ -25,10 +25,9 @@ int series_apply(const ChainView& v, const double* phi, const float2* in, float2
 int series_cg(hmc_ctx* c, const double* phi, const double2* chi, double2* x, double tol,
               int max_iter, cudaStream_t s);
 int series_trajectory(hmc_ctx* c, const TrajArgs& a, cudaStream_t s);
-// The series' batch kernel (kSeriesThreads threads, as many bytes of shared memory as *smem
-// receives); null on a CUDA error.
-const void* series_batch_kernel(unsigned* smem);
-constexpr int kSeriesThreads = 640;
+// The series' batch kernel, its threads and the bytes of shared memory a CTA has for
+// it; null on a CUDA error.
+const void* series_batch_kernel(unsigned* smem, int* threads);
 
 struct TcBatch;
 int tc_batch_create(const hmc_params* p, int n, TcBatch** out);
