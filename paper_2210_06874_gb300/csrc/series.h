@@ -54,6 +54,12 @@ HMC_HD inline bool series_pays64(int V, int k64, bool solve) {
     return V > 32 && 2 * k64 <= (solve ? 13 : 14) * ((V + 31) / 32);
 }
 
+// The message numbers of a launch start after `first`: 0 for a cluster, whose boxes
+// are cleared before each launch (a number that had come round to 0 would match a
+// cleared box), else where the context's last launch ended -- the boxes in global
+// memory then hold numbers just before it, also when it comes round.
+HMC_HD inline unsigned series_first(bool cluster, unsigned last) { return cluster ? 0u : last; }
+
 // Whether a CG vector of S slices of V sites (8 bytes each) still fits a shared
 // memory of `bytes` whose first `top` are taken.  In 64 bits: one CTA may own 2^30
 // site-slices.

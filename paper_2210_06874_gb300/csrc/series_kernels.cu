@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kApplyThreads)
 }
 
 // Per-launch set-up of a persistent kernel's team and workspace: the cluster's
-// mail boxes cleared before any member can write to them, the sequence number
+// mail boxes cleared before any member can write to them, or the sequence number
 // taken up where the context's last launch left it.
 struct Launch {
     int cluster;        // the grid is one cluster of this many CTAs (0: global team)
@@ -70,7 +70,7 @@ __device__ __forceinline__ bool begin(const ChainView& c, const Launch& la, Clus
     wk.mail_V = la.cluster ? c.V : 0;
     wk.norm_smem = norm;
     wk.seq = seq;
-    if (threadIdx.x == 0) *seq = *c.ser_seq;
+    if (threadIdx.x == 0) *seq = series_first(la.cluster != 0, *c.ser_seq);
     if (la.cluster) {
         uint64_t* m = reinterpret_cast<uint64_t*>(ser_dyn);
         for (int i = threadIdx.x; i < (int)(mail_bytes(c.V) / 8); i += blockDim.x) m[i] = 0;
@@ -86,8 +86,8 @@ __device__ __forceinline__ bool begin(const ChainView& c, const Launch& la, Clus
     __syncthreads();
     return true;
 }
-// No member leaves while others may still write to it; the context's next
-// launch starts past every number any CTA can have used.
+// No member leaves while others may still write to it; the context's next launch
+// with its mail in global memory starts past every number any CTA can have used.
 __device__ __forceinline__ void end(const ChainView& c, const Launch& la, const Work& wk) {
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) *c.ser_seq = *wk.seq + 16u;
