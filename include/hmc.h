@@ -401,14 +401,14 @@ int hmc_cg_solve_noalloc(const double* E, int L, int Nt, const double* phi, cons
  * one never completes and its bounded wait runs out.  0 restores normal
  * operation.
  *
- * hmc_debug_withhold: the same for the waits inside the FP32 iterations of the
+ * hmc_debug_misnumber: the same for the waits inside the FP32 iterations of the
  * automatic operand mode's series, which the padding never reaches: the team's
- * first CTA keeps to itself what (a sum of 1: its norms, 2: its boundary slices
- * of M^dag, 4: those of M) names, and its peers' waits for them run out.  0
- * restores normal operation.  No effect on a team of one CTA. */
+ * first CTA numbers its norms and boundary slices `ahead` (0..1024) half
+ * iterations ahead of the others, so from 16 on the waits for them, and its own,
+ * run out.  0 restores normal operation.  No effect on a team of one CTA. */
 int hmc_ctx_set_wait_limit(hmc_ctx* ctx, double seconds);
 int hmc_debug_team_padding(hmc_ctx* ctx, int extra_ctas);
-int hmc_debug_withhold(hmc_ctx* ctx, int what);
+int hmc_debug_misnumber(hmc_ctx* ctx, int ahead);
 
 /* Library version string (static storage). */
 const char* hmc_version(void);

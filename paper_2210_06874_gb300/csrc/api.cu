@@ -403,9 +403,9 @@ int hmc_debug_team_padding(hmc_ctx* c, int extra_ctas) {
     return HMC_OK;
 }
 
-int hmc_debug_withhold(hmc_ctx* c, int what) {
-    if (!c || what < 0 || what > 7) return HMC_ERR_BAD_ARG;
-    c->view.withhold = what;
+int hmc_debug_misnumber(hmc_ctx* c, int ahead) {
+    if (!c || ahead < 0 || ahead > 1024) return HMC_ERR_BAD_ARG;
+    c->view.misnumber = ahead;
     return HMC_OK;
 }
 

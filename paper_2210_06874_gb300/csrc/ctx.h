@@ -65,8 +65,8 @@ struct ChainView {
     uint64_t* slots;            // [kMaxTeam][kSlotWords] tagged partial sums
     int team_pad;               // testing only: CTAs every team barrier expects
                                 // beyond those launched (0 in normal use)
-    int withhold;               // testing only: what rank 0 of a series team keeps to
-                                // itself (1: norms, 2, 4: boundary slices; 0 in normal use)
+    int misnumber;              // testing only: rank 0 of a series team numbers its messages
+                                // this far ahead of the others (0 in normal use)
 };
 
 // The control block of a chain: uint64 wait limit, int status (+ 4 unused

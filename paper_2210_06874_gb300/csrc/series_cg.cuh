@@ -97,17 +97,14 @@ struct Link {
     uint64_t* norm;    // [2 kinds][T] every 16 words (global) or [2][16] (own shared memory)
 
     // msg: [2 kinds][T][V] x 2 words (global) or [2][mail_V] x 2 (shared memory)
-    // withhold (see ChainView): a boundary slice of rank 0 goes into its own box
-    // instead of its neighbour's
     __device__ __forceinline__ void init(const Team& tm, int V, int mail_V, uint64_t* msg,
-                                         uint64_t* nrm, int withhold) {
+                                         uint64_t* nrm) {
         T = tm.size;
         rank = tm.rank;
         cluster = tm.cs != nullptr;
         norm = nrm;
-        int dst[2] = {rank == 0 ? T - 1 : rank - 1, rank == T - 1 ? 0 : rank + 1};
+        const int dst[2] = {rank == 0 ? T - 1 : rank - 1, rank == T - 1 ? 0 : rank + 1};
         for (int k = 0; k < 2; ++k) {
-            if (rank == 0 && (withhold & (2 << k))) dst[k] = rank;
             if (cluster) {
                 own_s[k] = cta_smem_u32(msg) + 16u * (uint32_t)(k * mail_V);
                 to_s[k] = peer(own_s[k], dst[k]);
@@ -380,7 +377,7 @@ struct Work {
 // The loop invariants of a segment (shared memory).
 struct Geo {
     int LL, Nt, S, t0, SB, stride, K, it_end, max_iter;
-    bool alone, posts;   // posts: the team gets this CTA's norms (see ChainView::withhold)
+    bool alone;
     float c0, rmax, stop, ru2;
     size_t g0;      // first element of the own slices in [Nt][V]
     int* status;
@@ -423,7 +420,6 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
         g.LL = c.V / 2;
         g.Nt = c.Nt;
         g.alone = tm.size == 1;
-        g.posts = !g.alone && !(tm.rank == 0 && (c.withhold & 1));
         g.t0 = t_lo(tm.rank, c.Nt, tm.size);
         g.S = t_lo(tm.rank + 1, c.Nt, tm.size) - g.t0;
         g.SB = min(sh.SB, g.S);
@@ -438,10 +434,9 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
         g.max_iter = max_iter;
         g.status = tm.status;
         if (tm.cs)
-            g.lk.init(tm, c.V, wk.mail_V, reinterpret_cast<uint64_t*>(ser_dyn), wk.norm_smem,
-                      c.withhold);
+            g.lk.init(tm, c.V, wk.mail_V, reinterpret_cast<uint64_t*>(ser_dyn), wk.norm_smem);
         else
-            g.lk.init(tm, c.V, 0, c.ser_mail, c.ser_norm, c.withhold);
+            g.lk.init(tm, c.V, 0, c.ser_mail, c.ser_norm);
     }
     if (threadIdx.x < kSerMax32) s_ratio[threadIdx.x] = c.ser.r32[threadIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nww = (blockDim.x >> 5) - 1;
@@ -548,7 +543,7 @@ __device__ __noinline__ int segment(const ChainView& c, const Team tm, const Wor
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
                 own = __shfl_sync(0xffffffffu, a, 0);
-                if (g.posts) g.lk.post(kind, own, seq);
+                if (!g.alone) g.lk.post(kind, own, seq);
             });
 #pragma unroll
             for (int j = 0; j < N; ++j)

@@ -70,7 +70,8 @@ __device__ __forceinline__ bool begin(const ChainView& c, const Launch& la, Clus
     wk.mail_V = la.cluster ? c.V : 0;
     wk.norm_smem = norm;
     wk.seq = seq;
-    if (threadIdx.x == 0) *seq = series_first(la.cluster != 0, *c.ser_seq);
+    if (threadIdx.x == 0) *seq = series_first(la.cluster != 0, *c.ser_seq) +
+                                    (blockIdx.x == 0 ? (unsigned)c.misnumber : 0u);
     if (la.cluster) {
         uint64_t* m = reinterpret_cast<uint64_t*>(ser_dyn);
         for (int i = threadIdx.x; i < (int)(mail_bytes(c.V) / 8); i += blockDim.x) m[i] = 0;

@@ -107,7 +107,7 @@ SIGNATURES = {
                                             ctypes.POINTER(hmc_cg_stats), _P]),
     "hmc_ctx_set_wait_limit": (ctypes.c_int, [_P, ctypes.c_double]),
     "hmc_debug_team_padding": (ctypes.c_int, [_P, ctypes.c_int]),
-    "hmc_debug_withhold": (ctypes.c_int, [_P, ctypes.c_int]),
+    "hmc_debug_misnumber": (ctypes.c_int, [_P, ctypes.c_int]),
 }
 
 
@@ -318,11 +318,11 @@ class Context:
         CTAs beyond those launched, so their bounded waits run out."""
         _check("hmc_debug_team_padding", self.lib.hmc_debug_team_padding(self._h, extra_ctas))
 
-    def debug_withhold(self, what):
-        """Testing only: the first CTA of a series team keeps its norms (1), its
-        boundary slices of M^dag (2) or of M (4) to itself, so its peers' bounded
-        waits for them run out (0: normal operation)."""
-        _check("hmc_debug_withhold", self.lib.hmc_debug_withhold(self._h, what))
+    def debug_misnumber(self, ahead):
+        """Testing only: the first CTA of a series team numbers its messages this
+        many half iterations ahead of the others, so the bounded waits for them
+        run out (0: normal operation)."""
+        _check("hmc_debug_misnumber", self.lib.hmc_debug_misnumber(self._h, ahead))
 
     def trajectory(self, phi, seed, traj_index, chain=0, allow_not_converged=False):
         self._field(phi, "phi", torch.float64)
