@@ -1659,6 +1659,9 @@ int tc_batch_trajectory(TcBatch* b, double* phi, uint64_t seed, uint64_t traj,
             return HMC_ERR_CUDA;
         cudaMemcpyAsync(b->d_call, b->h_call, sizeof(tc::BatchCallArgs), cudaMemcpyHostToDevice, s);
         cudaMemsetAsync(b->d_queue, 0, sizeof(int), s);
+        // (a chain that no CTA gets to, once every one of them has failed, reports
+        // no solves instead of the last call's results)
+        cudaMemsetAsync(b->d_outs, 0, sizeof(double) * kNumScalars * b->n, s);
         {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(b->grid);
