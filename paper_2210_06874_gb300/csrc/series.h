@@ -54,6 +54,28 @@ HMC_HD inline bool series_pays64(int V, int k64, bool solve) {
     return V > 32 && 2 * k64 <= (solve ? 13 : 14) * ((V + 31) / 32);
 }
 
+// Whether a solve or trajectory of Nt slices of LL cells, which could have T CTAs,
+// runs on one cluster (of at most 16).  A global team's CTAs hold fewer cells, but
+// its exchange grows with T, as every CTA reads every other's word.  Milliseconds of
+// a solve to 1e-10 on one cluster / a global team, by the cells a CTA is spared:
+//   T = 18    81 (L = 9) 1.38 / 1.42   100 (10) 1.35 / 1.35   144 (12) 1.66 / 1.57
+//   T = 24    81 (9) 1.60 / 1.69       121 (11) 1.73 / 1.71   144 (12) 1.82 / 1.69
+//   T = 36   128 (8) 1.87 / 1.92       162 (9) 2.24 / 2.10    288 (12) 2.88 / 2.37
+//   T = 64   108 (6) 2.88 / 3.00       192 (8) 2.55 / 2.51    432 (12) 5.03 / 3.54
+//   T = 96   180 (6) 3.67 / 3.74       245 (7) 2.89 / 2.61
+//   T = 128  252 (6) 5.71 / 6.26       343 (7) 3.43 / 3.09
+//   T = 150  324 (6) 7.20 / 7.38
+// (trajectories the same to 2 %).  With at most 16 CTAs either way the cluster is
+// ahead (5 to 15 %) up to 324 cells a CTA and level at 576; beyond 608 a thread has
+// two cells.
+constexpr int kSerCluster = 16;
+HMC_HD inline bool series_on_cluster(int LL, int Nt, int T) {
+    const int Tc = T < kSerCluster ? T : kSerCluster;
+    if (Tc < 2) return false;
+    const long long S = (Nt + Tc - 1) / Tc, Sg = (Nt + T - 1) / T;
+    return S * LL <= 600 && 4 * (S - Sg) * LL <= (T > kSerCluster ? 300 + 7 * T : 0);
+}
+
 // The message numbers of a launch start after `first`: 0 for a cluster, whose boxes
 // are cleared before each launch (a number that had come round to 0 would match a
 // cleared box), else where the context's last launch ended -- the boxes in global

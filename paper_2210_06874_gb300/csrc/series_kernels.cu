@@ -247,8 +247,8 @@ int series_apply(const ChainView& v, const double* phi, const float2* in, float2
     return cudaGetLastError() == cudaSuccess ? HMC_OK : HMC_ERR_CUDA;
 }
 
-// Launch a persistent series kernel.  Teams of at most 16 CTAs go out as one
-// thread-block cluster, larger ones as a cooperative launch with global mail.
+// Launch a persistent series kernel: as one thread-block cluster where that is the
+// quicker (series_on_cluster), else as a cooperative launch with global mail.
 static int launch_series(hmc_ctx* c, const void* fn, tc::PersistentArgs& pa, ser::Launch& la,
                          void** args, cudaStream_t s) {
     const ChainView& v = c->view;
@@ -256,12 +256,8 @@ static int launch_series(hmc_ctx* c, const void* fn, tc::PersistentArgs& pa, ser
     if (c->params.team_ctas > 0) most = std::min(most, c->params.team_ctas);
     if (c->params.inner_ctas > 0) most = std::min(most, c->params.inner_ctas);
     int T = most;
-    // one cluster of 16 while a CTA keeps at most kClusterCells cells
-    constexpr int kClusterCells = 600;
-    const int Tc = std::min(most, 16);
-    bool cluster = Tc > 1 && ser::max_slices(v.Nt, Tc) * (v.V / 2) <= kClusterCells &&
-                   v.team_pad == 0;
-    if (cluster) T = Tc;
+    bool cluster = series_on_cluster(v.V / 2, v.Nt, most) && v.team_pad == 0;
+    if (cluster) T = std::min(most, kSerCluster);
     for (;;) {
         la.cluster = cluster ? T : 0;
         pa.inner = T;

@@ -1,7 +1,7 @@
 """Where the FP64 path takes the polynomial of the sparse hopping and where the
-dense E (csrc/series.h, series_pays64), on the CPU: the lattices and degrees that
-were measured on both sides; and, on the GPU, both forms against the oracle right
-at the line."""
+dense E (csrc/series.h, series_pays64), and where the mixed path takes one cluster
+and where a global-memory team (series_on_cluster), on the CPU: the sizes that were
+measured on both sides; and, on the GPU, both sides right at the lines."""
 import os
 import shutil
 import subprocess
@@ -19,6 +19,10 @@ MAIN = r"""
 #include <stdio.h>
 #include <stdlib.h>
 int main(int n, char** v) {
+    if (n == 4) {
+        printf("%%d\n", hmc::series_on_cluster(atoi(v[1]), atoi(v[2]), atoi(v[3])) ? 1 : 0);
+        return 0;
+    }
     for (int i = 1; i + 1 < n; i += 2) {
         hmc::HopSeries s;
         const int L = atoi(v[i]);
@@ -37,16 +41,56 @@ MEASURED = [(2, 0.125, 0, 0), (3, 0.125, 0, 0), (4, 0.25, 0, 0),
             (12, 1.3, 1, 1)]
 
 
-def test_rule_takes_the_measured_side(tmp_path):
+# (L, Nt, CTAs there could be, cluster)
+CLUSTER = [(3, 8, 8, 1), (6, 32, 32, 1), (6, 64, 64, 1), (8, 48, 48, 1), (6, 96, 96, 1),
+           (6, 128, 128, 1), (6, 150, 150, 1), (9, 24, 24, 1), (8, 36, 36, 1), (3, 200, 152, 1),
+           (16, 16, 16, 1), (20, 16, 16, 1), (9, 48, 48, 0), (9, 36, 36, 0), (8, 64, 64, 0),
+           (12, 18, 18, 0), (11, 24, 24, 0), (12, 32, 32, 0), (9, 64, 64, 0), (12, 48, 48, 0),
+           (16, 32, 32, 0), (7, 96, 96, 0), (7, 128, 128, 0), (12, 64, 64, 0), (24, 96, 96, 0),
+           (27, 3, 3, 0), (6, 32, 3, 1), (9, 20, 1, 0)]
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
     cxx = shutil.which("g++")
     if not cxx:
         pytest.skip("no g++")
-    (tmp_path / "m.cpp").write_text(MAIN % ROOT)
-    subprocess.run([cxx, "-O2", "-o", str(tmp_path / "m"), str(tmp_path / "m.cpp")], check=True)
-    args = [repr(a) for L, dk, *_ in MEASURED for a in (L, dk)]
-    out = subprocess.run([str(tmp_path / "m")] + args, check=True, capture_output=True,
-                         text=True).stdout.split()
-    assert [int(o) for o in out] == [s for m in MEASURED for s in m[2:]]
+    d = tmp_path_factory.mktemp("rule")
+    (d / "m.cpp").write_text(MAIN % ROOT)
+    subprocess.run([cxx, "-O2", "-o", str(d / "m"), str(d / "m.cpp")], check=True)
+
+    def run(*args):
+        return [int(w) for w in subprocess.run([str(d / "m"), *map(repr, args)], check=True,
+                                               capture_output=True, text=True).stdout.split()]
+    return run
+
+
+def test_rule_takes_the_measured_side(program):
+    out = program(*[a for L, dk, *_ in MEASURED for a in (L, dk)])
+    assert out == [s for m in MEASURED for s in m[2:]]
+
+
+@pytest.mark.parametrize("L,Nt,T,cluster", CLUSTER)
+def test_cluster_or_global_team(program, L, Nt, T, cluster):
+    assert program(L * L, Nt, T) == [cluster]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("L,Nt", [(8, 48), (9, 48), (6, 128), (8, 64), (9, 33), (24, 17)])
+def test_mixed_solves_around_the_cluster_line(L, Nt):
+    """Clusters and global teams, even and uneven slices: the FP64 path's residual of
+    the mixed solution (1e-10 asked for), and the same bits a second time."""
+    V, U, delta = 2 * L * L, 2.0, 0.125
+    c = hmc.Context(hmc.Params(L=L, Nt=Nt, beta=delta * Nt, U=U, precision=hmc.PREC_MIXED))
+    E = ops.transfer_matrix(lattice.hopping_matrix(L), delta)
+    phi = synth.gaussian_field(503, Nt, V, delta * U, scale=0.3)
+    chi = synth.complex_gaussian(504, Nt, V)
+    tphi, tchi = torch.from_numpy(phi).cuda(), torch.from_numpy(chi).cuda()
+    x, st = c.cg_solve(tphi, tchi, tol=1e-10, prec=hmc.PREC_MIXED)
+    r = chi - ops.apply_MMdag(E, phi, x.cpu().numpy())
+    assert st.status == 0 and np.linalg.norm(r) < 1.2e-10 * np.linalg.norm(chi)
+    y, _ = c.cg_solve(tphi, tchi, tol=1e-10, prec=hmc.PREC_MIXED)
+    assert torch.equal(x, y)
 
 
 @pytest.mark.gpu
