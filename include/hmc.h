@@ -89,11 +89,15 @@ typedef struct hmc_params {
                             those chains go first), 1 on one CTA, 0 on one
                             CTA or, where that shortens the step and every
                             chain is on the automatic operand mode, on a
-                            cluster of 8 (chains of over 2048 sites) */
+                            cluster of 8 (chains of over 2048 sites).  One chain
+                            of a batch without the series (see operand_mode)
+                            puts every chain of it on tensor-core tiles */
     int tile_slices;     /* time slices per tensor-core tile, one of 8, 16, 32
                             (operand_mode 4: 1..64; 0: automatic) */
     int inner_ctas;      /* CTAs running the FP32 iterations of the mixed CG
-                            (0: automatic; the FP64 steps use all CTAs) */
+                            (0: automatic).  Tensor-core tiles: the FP64 steps
+                            use all CTAs.  The automatic mode's series runs both
+                            on the same CTAs: a cap on the launch, like team_ctas */
     int operand_mode;    /* mixed path: 0 automatic (E as a polynomial of the
                             sparse hopping on CTAs that own time slices, where
                             3 |delta kappa| <= 4, V <= 1536, cluster_mode = 0 and

@@ -28,8 +28,8 @@
 // threads): contraction 5,100, wait for the neighbour and the norm 2,000,
 // epilogue 900, norm and scalars 600; at L = 6, Nt = 32 (a cluster of 16)
 // 2,600, 900, 470 and 490.  One CG iteration, tensor-core tiles -> here: L = 24
-// 41 us (split-K tiles 20) -> 8; L = 12, Nt = 64 20 -> 6.8; L = 6, Nt = 32 19 ->
-// 4.5.
+// 41 us (split-K tiles 20) -> 8; L = 12, Nt = 64 20 -> 4.8 (64 CTAs; 6.4 on one
+// cluster); L = 6, Nt = 32 19 -> 3.8-4.0.
 #pragma once
 
 #include "cg_scalars.cuh"
